@@ -11,8 +11,7 @@
 // boxes that do not touch (dist > 0), the block list.  Device: one CTA per admissible block runs the cross approximation on the
 // resident dense matrix (rows and columns gathered through the cluster permutation), blocks whose
 // crosses reach the rank cap, or would take at least the block's own entries, stay dense, and the factors and dense blocks are packed into one
-// buffer per matrix.  The product y = H x gathers x into cluster order, runs one CTA per (block,
-// column) with FP64 accumulation and FP64 atomics into y, and scatters back.
+// buffer per matrix.  The product y = H x (FP64 accumulation) runs over cross items and row tiles.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -158,10 +157,11 @@ constexpr unsigned FULL = 0xffffffffu;
 
 // one block of the compressed form: rows [r0, r1) and columns [c0, c1) in cluster order; rank < 0
 // for a dense block (m x n row-major at off), else U (rank x m, one cross per row of U) at off and
-// Vt (rank x n) at off + rank m
+// Vt (rank x n) at off + rank m; t0: its first entry of a product's cross sums (rank of Vt x, rank
+// of U x)
 struct HmBlockDev {
   int32_t r0, r1, c0, c1;
-  int32_t rank, pad;
+  int32_t rank, t0;
   long long off;
 };
 
@@ -380,133 +380,204 @@ __global__ void __launch_bounds__(HM_THREADS)
   }
 }
 
-// xp (n x nrhs, cluster order) = x gathered through perm
+// ---- the product y = H x ----
+// Three launches per group of columns (at most HM_COLS columns a group):
+//   hm_gather   x into cluster order, the columns of a group interleaved
+//   hm_cross    t = Vt x[c0..c1) and t' = U x[r0..r1) of every low-rank block, one warp per four
+//               crosses of one side, so an x entry is read once for four crosses
+//   hm_rows     y of one tile of at most 32 rows per CTA: every block that covers the tile adds U t
+//               (or Vt^T t' below the diagonal, or its dense entries), lane = row, the blocks dealt to
+//               the CTA's warps; one store per row through the permutation
+// Every stored entry is used once per side, so no sum crosses a CTA: no atomics, no zeroed output,
+// and a product is the same bits on every run.  Bound: the FP64 pipe (2 lanes per clock and SM, 90 to
+// 93 % busy), 8 multiply-adds per stored entry and column; the FP32 entries are widened with integer
+// operations, which keeps the conversions off that pipe.  Measured on GB300: both products of an
+// ellipsoid of 17280 functions and 11520 cells (47.8 M stored entries), 8 columns: 10.3 ms; one CTA
+// per block and column with a row a thread and FP64 atomics took 20.2 ms.
+constexpr int HM_COLS = 4;        // columns of a group
+constexpr int HM_TILE = 32;       // rows of a tile (one lane each)
+constexpr int HM_CROSS = 4;       // crosses of one warp's item
+constexpr int HM_CROSS_THREADS = 128;
+constexpr int HM_ROW_WARPS = HM_THREADS / 32;
+constexpr size_t HM_SCRATCH = (size_t)256 << 20;  // cross sums of one pass over the columns
+
+struct HmTile {
+  int32_t row0, rows;      // rows [row0, row0 + rows) in cluster order
+  int32_t begin, end;      // its entries of the cover list: 2 block + (1: as columns)
+};
+
+// FP32 -> FP64 by moving the bits: exponent rebased by 896, mantissa shifted by 29.  Zeros,
+// subnormals, infinities and NaN take the conversion instruction.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f);
+  if ((u & 0x7f800000u) - 0x00800000u >= 0x7f000000u) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// xp: group g (columns 4 g ..) at 4 g n, entry p, column c of the group at p * (columns of the group) + c
 __global__ void hm_gather_kernel(const double2* __restrict__ x, const int32_t* __restrict__ perm, int n, int nrhs,
                                  double2* __restrict__ xp) {
   RF_COUNT_LAUNCH();
   const long long total = (long long)n * nrhs;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
-    const long long c = e / n;
-    const int p = (int)(e - c * n);
-    xp[e] = x[c * n + perm[p]];
+    const int c = (int)(e / n), p = (int)(e - (long long)c * n);
+    const int g = c / HM_COLS, nc = min(HM_COLS, nrhs - g * HM_COLS);
+    xp[(size_t)g * HM_COLS * n + (size_t)p * nc + (c - g * HM_COLS)] = x[(size_t)c * n + perm[p]];
   }
 }
 
-// y (original order) = yp scattered through perm
-__global__ void hm_scatter_kernel(const double2* __restrict__ yp, const int32_t* __restrict__ perm, int n, int nrhs,
-                                  double2* __restrict__ y) {
+// Warp sums of V = 2^k values a lane: afterwards v[0] of lane l is the sum of value l * V / 32 (each
+// exchange halves the values a lane holds: V - 1 + max(0, 5 - k) additions instead of 5 V).
+template <int V>
+__device__ __forceinline__ void warp_sums(double (&v)[V], int lane) {
+#pragma unroll
+  for (int step = 0; step < 5; ++step) {
+    const int off = 16 >> step, h = V >> (step + 1);
+    if (h == 0) {
+      v[0] += __shfl_xor_sync(FULL, v[0], off);
+    } else {
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int k = 0; k < h; ++k) {
+        const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+        v[k] = keep + __shfl_xor_sync(FULL, send, off);
+      }
+    }
+  }
+}
+
+// t[(l0 + q) nrhs + c] = sum_j f[q len + j] x[j NC + c] for q < nl crosses (NC columns)
+template <int NC>
+__device__ __forceinline__ void cross_dots(const float2* __restrict__ f, int len, int nl, const double2* __restrict__ x,
+                                           double2* __restrict__ t, int nrhs, int lane) {
+  constexpr int V = HM_CROSS * (NC == 3 ? 4 : NC) * 2;
+  double acc[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) acc[k] = 0.0;
+  for (int j = lane; j < len; j += 32) {
+    double2 xv[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) xv[c] = x[(size_t)j * NC + c];
+#pragma unroll
+    for (int q = 0; q < HM_CROSS; ++q) {
+      const float2 e = q < nl ? f[(size_t)q * len + j] : make_float2(0.f, 0.f);
+      if (q >= nl) continue;
+      const double er = widen(e.x), ei = widen(e.y);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        double& re = acc[(q * (NC == 3 ? 4 : NC) + c) * 2];
+        double& im = acc[(q * (NC == 3 ? 4 : NC) + c) * 2 + 1];
+        re = fma(er, xv[c].x, fma(-ei, xv[c].y, re));
+        im = fma(er, xv[c].y, fma(ei, xv[c].x, im));
+      }
+    }
+  }
+  warp_sums<V>(acc, lane);
+  if (V < 32 && (lane & (32 / V - 1))) return;
+  const int v = lane * V / 32, q = v / (V / HM_CROSS), c = (v / 2) % (V / HM_CROSS / 2);
+  if (q < nl && c < NC) reinterpret_cast<double*>(t + (size_t)q * nrhs + c)[v & 1] = acc[0];
+}
+
+// items: x = 2 block + (1: U, the row side), y = first cross
+__global__ void __launch_bounds__(HM_CROSS_THREADS)
+    hm_cross_kernel(const HmBlockDev* __restrict__ blk, const int2* __restrict__ items, int nitems,
+                    const float2* __restrict__ H, const double2* __restrict__ xp, double2* __restrict__ t, int n,
+                    int nrhs) {
   RF_COUNT_LAUNCH();
-  const long long total = (long long)n * nrhs;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long c = e / n;
-    const int p = (int)(e - c * n);
-    y[c * n + perm[p]] = yp[e];
+  const int it = blockIdx.x * (HM_CROSS_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (it >= nitems) return;
+  const int2 item = items[it];
+  const HmBlockDev B = blk[item.x >> 1];
+  const int side = item.x & 1, m = B.r1 - B.r0, nn = B.c1 - B.c0, len = side ? m : nn;
+  const int g = blockIdx.y * HM_COLS, nc = min(HM_COLS, nrhs - g), nl = min(HM_CROSS, B.rank - item.y);
+  const float2* f = H + B.off + (side ? 0 : (size_t)B.rank * m) + (size_t)item.y * len;
+  const double2* x = xp + (size_t)g * n + (size_t)(side ? B.r0 : B.c0) * nc;
+  double2* o = t + ((size_t)B.t0 + (side ? B.rank : 0) + item.y) * nrhs + g;
+  switch (nc) {
+    case 1: return cross_dots<1>(f, len, nl, x, o, nrhs, lane);
+    case 2: return cross_dots<2>(f, len, nl, x, o, nrhs, lane);
+    case 3: return cross_dots<3>(f, len, nl, x, o, nrhs, lane);
+    default: return cross_dots<4>(f, len, nl, x, o, nrhs, lane);
   }
 }
 
-__device__ __forceinline__ void atomic_add_c(double2* p, double re, double im) {
-  atomicAdd(&p->x, re);
-  atomicAdd(&p->y, im);
-}
-
-__device__ __forceinline__ void warp_sum2(double& a, double& b) {
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(FULL, a, o);
-    b += __shfl_down_sync(FULL, b, o);
+template <int NC>
+__device__ __forceinline__ void madd(double (&acc)[2 * HM_COLS], float2 e, const double2* __restrict__ x) {
+  const double er = widen(e.x), ei = widen(e.y);
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const double2 v = x[c];
+    acc[2 * c] = fma(er, v.x, fma(-ei, v.y, acc[2 * c]));
+    acc[2 * c + 1] = fma(er, v.y, fma(ei, v.x, acc[2 * c + 1]));
   }
 }
 
-// yp += H xp for one block and one column (grid: blocks x columns), FP64 accumulation.  A block
-// off the block diagonal adds its transpose too: y[c0..c1) += B^T x[r0..r1).
+// the sums of one row (row0 + lane) of a tile over the cover entries begin + w, begin + w + 8, ...
+template <int NC>
+__device__ __forceinline__ void tile_rows(const HmTile& T, const int32_t* __restrict__ cover,
+                                          const HmBlockDev* __restrict__ blk, const float2* __restrict__ H,
+                                          const double2* __restrict__ xg, const double2* __restrict__ t, int nrhs,
+                                          int w, int lane, double (&acc)[2 * HM_COLS]) {
+  const bool live = lane < T.rows;
+  for (int q = T.begin + w; q < T.end; q += HM_ROW_WARPS) {
+    const int code = cover[q];
+    const HmBlockDev B = blk[code >> 1];
+    const int cols = code & 1, m = B.r1 - B.r0, nn = B.c1 - B.c0;
+    const int i = T.row0 + (live ? lane : 0) - (cols ? B.c0 : B.r0);
+    const float2* M = H + B.off;
+    if (B.rank >= 0) {  // U t, or Vt^T t' below the diagonal
+      const int len = cols ? nn : m;
+      const float2* f = M + (cols ? (size_t)B.rank * m : 0) + i;
+      const double2* tb = t + ((size_t)B.t0 + (cols ? B.rank : 0)) * nrhs;
+#pragma unroll 4
+      for (int l = 0; l < B.rank; ++l) madd<NC>(acc, f[(size_t)l * len], tb + (size_t)l * nrhs);
+    } else if (cols) {  // the transpose of a dense block
+      const double2* x = xg + (size_t)B.r0 * NC;
+#pragma unroll 4
+      for (int p = 0; p < m; ++p) madd<NC>(acc, M[(size_t)p * nn + i], x + (size_t)p * NC);
+    } else if (B.r0 == B.c0) {  // a diagonal block is symmetric: read it along its rows
+      const double2* x = xg + (size_t)B.c0 * NC;
+#pragma unroll 4
+      for (int j = 0; j < nn; ++j) madd<NC>(acc, M[(size_t)j * nn + i], x + (size_t)j * NC);
+    } else {
+      const double2* x = xg + (size_t)B.c0 * NC;
+#pragma unroll 4
+      for (int j = 0; j < nn; ++j) madd<NC>(acc, M[(size_t)i * nn + j], x + (size_t)j * NC);
+    }
+  }
+}
+
 __global__ void __launch_bounds__(HM_THREADS)
-    hm_apply_kernel(const HmBlockDev* __restrict__ blk, const float2* __restrict__ H, const double2* __restrict__ xp,
-                    double2* __restrict__ yp, int n) {
+    hm_rows_kernel(const HmTile* __restrict__ tiles, const int32_t* __restrict__ cover,
+                   const HmBlockDev* __restrict__ blk, const float2* __restrict__ H, const double2* __restrict__ xp,
+                   const double2* __restrict__ t, const int32_t* __restrict__ perm, double2* __restrict__ y, int n,
+                   int nrhs) {
   RF_COUNT_LAUNCH();
-  __shared__ double2 t[HM_MAX_RANK];
-  const HmBlockDev B = blk[blockIdx.x];
-  const int m = B.r1 - B.r0, nn = B.c1 - B.c0, tid = threadIdx.x;
-  const double2* xc = xp + (size_t)blockIdx.y * n;
-  double2* yc = yp + (size_t)blockIdx.y * n;
-  const bool mirror = B.r0 != B.c0;
-  const float2* M = H + B.off;
-  if (B.rank < 0) {
-    for (int i = tid; i < m; i += HM_THREADS) {
-      double a = 0.0, b = 0.0;
-      const float2* row = M + (size_t)i * nn;
-      for (int j = 0; j < nn; ++j) {
-        const float2 d = row[j];
-        const double2 v = xc[B.c0 + j];
-        a += (double)d.x * v.x - (double)d.y * v.y;
-        b += (double)d.x * v.y + (double)d.y * v.x;
-      }
-      atomic_add_c(yc + B.r0 + i, a, b);
-    }
-    if (mirror) {
-      for (int j = tid; j < nn; j += HM_THREADS) {
-        double a = 0.0, b = 0.0;
-        for (int i = 0; i < m; ++i) {
-          const float2 d = M[(size_t)i * nn + j];
-          const double2 v = xc[B.r0 + i];
-          a += (double)d.x * v.x - (double)d.y * v.y;
-          b += (double)d.x * v.y + (double)d.y * v.x;
-        }
-        atomic_add_c(yc + B.c0 + j, a, b);
-      }
-    }
-    return;
+  __shared__ double part[HM_ROW_WARPS][2 * HM_COLS][HM_TILE];
+  const HmTile T = tiles[blockIdx.x];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = blockIdx.y * HM_COLS, nc = min(HM_COLS, nrhs - g);
+  const double2* xg = xp + (size_t)g * n;
+  double acc[2 * HM_COLS];
+#pragma unroll
+  for (int k = 0; k < 2 * HM_COLS; ++k) acc[k] = 0.0;
+  switch (nc) {
+    case 1: tile_rows<1>(T, cover, blk, H, xg, t + g, nrhs, w, lane, acc); break;
+    case 2: tile_rows<2>(T, cover, blk, H, xg, t + g, nrhs, w, lane, acc); break;
+    case 3: tile_rows<3>(T, cover, blk, H, xg, t + g, nrhs, w, lane, acc); break;
+    default: tile_rows<4>(T, cover, blk, H, xg, t + g, nrhs, w, lane, acc); break;
   }
-  const int r = B.rank, w = tid >> 5, lane = tid & 31;
-  const float2* U = M;
-  const float2* Vt = M + (size_t)r * m;
-  // t = Vt x[c0..c1), one warp per cross
-  for (int l = w; l < r; l += HM_THREADS / 32) {
-    double a = 0.0, b = 0.0;
-    for (int j = lane; j < nn; j += 32) {
-      const float2 v = Vt[(size_t)l * nn + j];
-      const double2 x = xc[B.c0 + j];
-      a += (double)v.x * x.x - (double)v.y * x.y;
-      b += (double)v.x * x.y + (double)v.y * x.x;
-    }
-    warp_sum2(a, b);
-    if (lane == 0) t[l] = make_double2(a, b);
-  }
+#pragma unroll
+  for (int k = 0; k < 2 * HM_COLS; ++k) part[w][k][lane] = acc[k];
   __syncthreads();
-  for (int i = tid; i < m; i += HM_THREADS) {
-    double a = 0.0, b = 0.0;
-    for (int l = 0; l < r; ++l) {
-      const float2 u = U[(size_t)l * m + i];
-      a += (double)u.x * t[l].x - (double)u.y * t[l].y;
-      b += (double)u.x * t[l].y + (double)u.y * t[l].x;
-    }
-    atomic_add_c(yc + B.r0 + i, a, b);
-  }
-  if (mirror) {
-    __syncthreads();  // t is rewritten
-    // t = U x[r0..r1) (the transpose: (U Vt)^T x = Vt^T (U^T x))
-    for (int l = w; l < r; l += HM_THREADS / 32) {
-      double a = 0.0, b = 0.0;
-      for (int i = lane; i < m; i += 32) {
-        const float2 u = U[(size_t)l * m + i];
-        const double2 x = xc[B.r0 + i];
-        a += (double)u.x * x.x - (double)u.y * x.y;
-        b += (double)u.x * x.y + (double)u.y * x.x;
-      }
-      warp_sum2(a, b);
-      if (lane == 0) t[l] = make_double2(a, b);
-    }
-    __syncthreads();
-    for (int j = tid; j < nn; j += HM_THREADS) {
-      double a = 0.0, b = 0.0;
-      for (int l = 0; l < r; ++l) {
-        const float2 v = Vt[(size_t)l * nn + j];
-        a += (double)v.x * t[l].x - (double)v.y * t[l].y;
-        b += (double)v.x * t[l].y + (double)v.y * t[l].x;
-      }
-      atomic_add_c(yc + B.c0 + j, a, b);
-    }
-  }
+  static_assert(HM_THREADS == 2 * HM_COLS * HM_TILE, "one thread per (value, row) of a tile");
+  const int k = threadIdx.x / HM_TILE, i = threadIdx.x % HM_TILE;
+  if (i >= T.rows || k >= 2 * nc) return;
+  double s = 0.0;
+#pragma unroll
+  for (int v = 0; v < HM_ROW_WARPS; ++v) s += part[v][k][i];
+  reinterpret_cast<double*>(y + (size_t)(g + k / 2) * n + perm[T.row0 + i])[k & 1] = s;
 }
 
 }  // namespace
@@ -518,6 +589,10 @@ struct HmPart {
   int32_t* perm = nullptr;       // cluster order -> original index (device)
   HmBlockDev* blocks = nullptr;  // (device)
   float2* data = nullptr;        // dense blocks and crosses (device)
+  int2* items = nullptr;         // cross items of the low-rank blocks, longest first (device)
+  HmTile* tiles = nullptr;       // row tiles (device)
+  int32_t* cover = nullptr;      // blocks over each tile (device)
+  int nitems = 0, ntiles = 0, ncross = 0;
   long long elems = 0;
   int64_t n_lowrank = 0, n_dense = 0, n_capped = 0, n_small = 0;
   int max_rank = 0;
@@ -543,6 +618,75 @@ struct HmTemps {
     return e;
   }
 };
+
+// What a product runs over.  Tiles: at most 32 rows that no block boundary cuts, each with the blocks
+// that cover it (2 block, + 1 where the tile lies in the block's columns).
+struct CoverLists {
+  std::vector<HmTile> tiles;
+  std::vector<int32_t> cover;
+};
+
+CoverLists cover_lists(const std::vector<HmBlockHost>& blk, int n) {
+  CoverLists L;
+  std::vector<uint8_t> cut((size_t)n + 1, 0);
+  for (const HmBlockHost& B : blk) cut[B.r0] = cut[B.r1] = cut[B.c0] = cut[B.c1] = 1;
+  std::vector<int32_t> first((size_t)n + 1, 0);  // first[p]: tiles that start below p
+  for (int p = 0; p < n;) {
+    int q = p + 1;
+    while (q < n && q - p < HM_TILE && !cut[q]) ++q;
+    for (int i = p + 1; i <= q; ++i) first[i] = (int32_t)L.tiles.size() + 1;
+    L.tiles.push_back({p, q - p, 0, 0});
+    p = q;
+  }
+  auto each = [&](auto&& f) {
+    for (size_t b = 0; b < blk.size(); ++b) {
+      const HmBlockHost& B = blk[b];
+      for (int i = first[B.r0]; i < first[B.r1]; ++i) f(i, (int32_t)(2 * b));
+      if (B.r0 != B.c0)
+        for (int i = first[B.c0]; i < first[B.c1]; ++i) f(i, (int32_t)(2 * b + 1));
+    }
+  };
+  each([&](int i, int32_t) { ++L.tiles[i].end; });
+  int32_t total = 0;
+  for (HmTile& t : L.tiles) {
+    const int32_t c = t.end;
+    t.begin = t.end = total;
+    total += c;
+  }
+  L.cover.resize(total);
+  each([&](int i, int32_t code) { L.cover[L.tiles[i].end++] = code; });
+  return L;
+}
+
+// The cross items of the low-rank blocks, the longest first (by binary order of magnitude), so that
+// the last ones to run are short.
+std::vector<int2> cross_items(const std::vector<HmBlockDev>& blk) {
+  size_t count[32] = {}, at[32], total = 0;
+  auto each = [&](auto&& f) {
+    for (size_t b = 0; b < blk.size(); ++b)
+      for (int side = 0; side < 2 && blk[b].rank > 0; ++side) {
+        int len = side ? blk[b].r1 - blk[b].r0 : blk[b].c1 - blk[b].c0, mag = 0;
+        for (; len > 1; len >>= 1) ++mag;
+        for (int l = 0; l < blk[b].rank; l += HM_CROSS) f(mag, make_int2((int)(2 * b) + side, l));
+      }
+  };
+  each([&](int mag, int2) { ++count[mag]; });
+  for (int mag = 31; mag >= 0; --mag) {
+    at[mag] = total;
+    total += count[mag];
+  }
+  std::vector<int2> items(total);
+  each([&](int mag, int2 v) { items[at[mag]++] = v; });
+  return items;
+}
+
+template <class T>
+cudaError_t keep(T** d, const std::vector<T>& h, std::vector<void*>& owned) {
+  cudaError_t e = dev_malloc(d, std::max<size_t>(h.size() * sizeof(T), 8));
+  if (e != cudaSuccess) return e;
+  owned.push_back(*d);
+  return h.empty() ? cudaSuccess : cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
+}
 
 // Compresses the dense n x n matrix A (row stride ld, both triangles stored) whose items have the
 // given centres and support boxes.  owned receives the part's device buffers; budget_left bounds
@@ -582,7 +726,10 @@ int build_part(const float2* A, int ld, int n, const std::vector<double>& cen, c
   std::vector<int32_t> rank(cand.size(), 0), status(cand.size(), 1);
   float2* slots = nullptr;
   long long* slot_d = nullptr;
-  if (!cand.empty()) {
+  CoverLists lists;
+  if (cand.empty()) {
+    lists = cover_lists(blocks, n);
+  } else {
     HmBlockDev* cand_d = nullptr;
     int32_t *rank_d = nullptr, *status_d = nullptr;
     HM_CUDA(tmp.alloc(&cand_d, cand.size() * sizeof(HmBlockDev)));
@@ -599,6 +746,7 @@ int build_part(const float2* A, int ld, int n, const std::vector<double>& cen, c
                                                           (float)o.eps, slots, rank_d, status_d);
     }
     HM_CUDA(cudaGetLastError());
+    lists = cover_lists(blocks, n);  // while the crosses are found
     HM_CUDA(cudaMemcpy(rank.data(), rank_d, 4 * cand.size(), cudaMemcpyDeviceToHost));
     HM_CUDA(cudaMemcpy(status.data(), status_d, 4 * cand.size(), cudaMemcpyDeviceToHost));
   }
@@ -619,6 +767,8 @@ int build_part(const float2* A, int ld, int n, const std::vector<double>& cen, c
         ++out.n_small;  // the crosses would take at least the block's own entries
       } else {
         d.rank = rank[c];
+        d.t0 = out.ncross;
+        out.ncross += 2 * d.rank;
         s = slot[c];
         ++out.n_lowrank;
         out.max_rank = std::max(out.max_rank, rank[c]);
@@ -643,8 +793,15 @@ int build_part(const float2* A, int ld, int n, const std::vector<double>& cen, c
     hm_pack_kernel<<<(unsigned)fin.size(), HM_THREADS>>>(A, ld, out.perm, out.blocks, fslot_d, cap, slots, out.data);
     HM_CUDA(cudaGetLastError());
   }
+  const std::vector<int2> items = cross_items(fin);
+  out.nitems = (int)items.size();
+  out.ntiles = (int)lists.tiles.size();
+  HM_CUDA(keep(&out.items, items, owned));
+  HM_CUDA(keep(&out.tiles, lists.tiles, owned));
+  HM_CUDA(keep(&out.cover, lists.cover, owned));
   HM_CUDA(cudaStreamSynchronize(0));
-  out.bytes = 8ull * (uint64_t)off + sizeof(HmBlockDev) * fin.size() + 4ull * n;
+  out.bytes = 8ull * (uint64_t)off + sizeof(HmBlockDev) * fin.size() + 4ull * n + sizeof(int2) * items.size() +
+              sizeof(HmTile) * lists.tiles.size() + 4ull * lists.cover.size();
   return RFCMP_OK;
 }
 
@@ -805,24 +962,32 @@ int rfcmp_hm_apply(rfcmp_hm* hm, int which, const rfcmp_c128* x, rfcmp_c128* y, 
         hm->nb_streams.push_back(st);
     }
   }
-  const long long total = (long long)P.n * nrhs;
-  if (total == 0) return RFCMP_OK;
-  double2 *xp = nullptr, *yp = nullptr;
-  HM_CUDA(cudaMallocAsync(&xp, 16 * (size_t)total, st));
-  cudaError_t e = cudaMallocAsync(&yp, 16 * (size_t)total, st);
-  if (e == cudaSuccess) {
+  if (P.n == 0) return RFCMP_OK;
+  // scratch: x in cluster order and the cross sums, at most HM_SCRATCH bytes of sums at a time
+  const size_t per_col = 16 * (size_t)std::max(P.ncross, 1);
+  const int64_t most = std::max<int64_t>(HM_COLS, (int64_t)(HM_SCRATCH / per_col) / HM_COLS * HM_COLS);
+  const int64_t width = std::min<int64_t>(nrhs, most);
+  double2* xp = nullptr;
+  HM_CUDA(cudaMallocAsync(&xp, (16 * (size_t)P.n + per_col) * (size_t)width, st));
+  double2* t = xp + (size_t)P.n * width;
+  for (int64_t c = 0; c < nrhs; c += width) {
+    const int nr = (int)std::min<int64_t>(width, nrhs - c);
+    const long long total = (long long)P.n * nr;
+    const unsigned groups = (unsigned)((nr + HM_COLS - 1) / HM_COLS);
     const int grid = (int)std::min<long long>((total + HM_THREADS - 1) / HM_THREADS, 152 * 8);
-    hm_gather_kernel<<<grid, HM_THREADS, 0, st>>>(reinterpret_cast<const double2*>(x), P.perm, P.n, (int)nrhs, xp);
-    e = cudaMemsetAsync(yp, 0, 16 * (size_t)total, st);
-    if (e == cudaSuccess && P.nblocks > 0) {
-      ProfScope prof("hm_apply", 8.0 * (double)P.elems + 32.0 * (double)total, 0.0, st);
-      hm_apply_kernel<<<dim3((unsigned)P.nblocks, (unsigned)nrhs), HM_THREADS, 0, st>>>(P.blocks, P.data, xp, yp, P.n);
+    hm_gather_kernel<<<grid, HM_THREADS, 0, st>>>(reinterpret_cast<const double2*>(x) + (size_t)c * P.n, P.perm, P.n,
+                                                  nr, xp);
+    ProfScope prof("hm_apply", 8.0 * (double)P.elems + 32.0 * (double)total, 16.0 * (double)P.elems * nr, st);
+    if (P.nitems > 0) {
+      const int per = HM_CROSS_THREADS / 32;
+      hm_cross_kernel<<<dim3((P.nitems + per - 1) / per, groups), HM_CROSS_THREADS, 0, st>>>(
+          P.blocks, P.items, P.nitems, P.data, xp, t, P.n, nr);
     }
-    if (e == cudaSuccess)
-      hm_scatter_kernel<<<grid, HM_THREADS, 0, st>>>(yp, P.perm, P.n, (int)nrhs, reinterpret_cast<double2*>(y));
-    if (e == cudaSuccess) e = cudaGetLastError();
-    cudaFreeAsync(yp, st);
+    hm_rows_kernel<<<dim3(P.ntiles, groups), HM_THREADS, 0, st>>>(P.tiles, P.cover, P.blocks, P.data, xp, t, P.perm,
+                                                                  reinterpret_cast<double2*>(y) + (size_t)c * P.n, P.n,
+                                                                  nr);
   }
+  cudaError_t e = cudaGetLastError();
   cudaFreeAsync(xp, st);
   if (e != cudaSuccess) return set_error(RFCMP_ERR_CUDA, std::string("rfcmp_hm_apply: ") + cudaGetErrorString(e));
   return RFCMP_OK;
