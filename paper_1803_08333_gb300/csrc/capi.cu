@@ -517,7 +517,7 @@ int ensure_workspace(rfcmp_op* op, int cols) {
     if (ex) {
       RF_TRY(dalloc(&ws->ms.xd, (size_t)EXACT_DIGITS * 2 * cols * ws->ms.cap_ld, ws->owned));
       RF_TRY(dalloc(&ws->ms.xe, (size_t)2 * cols, ws->owned));
-      RF_TRY(dalloc(&ws->ms.D64, (size_t)4 * cols * capn, ws->owned));
+      RF_TRY(dalloc(&ws->ms.D64, exact_result_doubles(cols) * capn, ws->owned));
     }
   }
   op->ws = std::move(ws);

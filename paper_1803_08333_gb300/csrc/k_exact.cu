@@ -29,11 +29,20 @@
 // accumulators alternate between K-blocks; warps 2..9 fold a finished K-block (two warps per
 // 32-lane quadrant of tensor memory, 16 columns each) while the next one accumulates, and write D.  Every wait
 // is bounded; on timeout the kernel records an error code, frees its tensor memory and returns.
+//
+// Up to XI_COLS columns D is the pair of integers (H, G) itself, scaled and combined by the kernel
+// after it.  The integer sums are exact, so the K range of a tile can be split over CTAs that add
+// theirs with 64-bit atomics (any order, the same bits): a matrix of few row tiles still fills the
+// chip.  16 columns on GB300: a factor of 5120 cells (40 tiles, split 3) 136 -> 66 us, V (80 tiles,
+// split 5) 160 -> 121 us, T_A of 7680 functions (120 tiles) unchanged at 237 us, where the digit
+// planes take 209 us to leave HBM.
 #include <cuda.h>
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstring>
 #include <mutex>
 
@@ -75,7 +84,8 @@ static_assert(XBN == 32, "two epilogue warps of 16 columns per tensor-memory qua
 
 __global__ void __launch_bounds__(XTHREADS, 1)
 exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, const int* __restrict__ ea,
-                  const int* __restrict__ eb, double* __restrict__ D, long long ldd, int* __restrict__ err) {
+                  const int* __restrict__ eb, double* __restrict__ D, longlong2* __restrict__ DI, long long ldd,
+                  int* __restrict__ err) {
   RF_COUNT_LAUNCH();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -86,8 +96,11 @@ exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, c
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n0 = blockIdx.x * XBN, m0 = blockIdx.y * BM;  // N tiles fastest: CTAs sharing A run together
-  const int ksteps = (K + XBK - 1) / XBK;
-  const int nkb = (ksteps + XSPK - 1) / XSPK;
+  const int all_steps = (K + XBK - 1) / XBK, all_kb = (all_steps + XSPK - 1) / XSPK;
+  // this CTA's K-blocks [kb0, kb1)
+  const int kb0 = (int)((long long)all_kb * blockIdx.z / gridDim.z);
+  const int kb1 = (int)((long long)all_kb * (blockIdx.z + 1) / gridDim.z);
+  const int step0 = kb0 * XSPK, ksteps = min(kb1 * XSPK, all_steps) - step0, nkb = kb1 - kb0;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < XSTAGES; ++s) {
@@ -120,7 +133,7 @@ exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, c
           break;
         }
         uint8_t* st = smem + s * XSTAGE;
-        const int kx = it * XBK;
+        const int kx = (step0 + it) * XBK;
         mbar_expect_tx(&full[s], XSTAGE);
 #pragma unroll
         for (int p = 0; p < XS; ++p) tma_load_2d(st + p * XTILE_A, &maps.a[p], &full[s], kx, m0);
@@ -181,6 +194,10 @@ exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, c
 #pragma unroll
       for (int L = 0; L < XS; ++L) tmem_ld16_async(base + (uint32_t)(L * XBN), r[L]);
       tmem_wait_ld();
+#pragma unroll
+      for (int L = 0; L < XS; ++L)  // no use of a loaded register may move before the wait
+#pragma unroll
+        for (int j = 0; j < 16; ++j) asm volatile("" : "+r"(r[L][j]));
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[buf]);  // the buffer may take the next K-block
@@ -193,7 +210,20 @@ exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, c
         G[j] += p[3] * 65536LL + p[4] * 256LL + p[5];
       }
     }
-    if (ok && row < M) {
+    if (ok && row < M && DI) {
+      longlong2* dst = DI + (size_t)row * ldd;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const int col = n0 + h + j;
+        if (col >= N) continue;
+        if (gridDim.z == 1) {
+          dst[col] = make_longlong2(H[j], G[j]);
+        } else {
+          atomicAdd(reinterpret_cast<unsigned long long*>(&dst[col].x), (unsigned long long)H[j]);
+          atomicAdd(reinterpret_cast<unsigned long long*>(&dst[col].y), (unsigned long long)G[j]);
+        }
+      }
+    } else if (ok && row < M) {
       const int er = ea[row];
       double* dst = D + (size_t)row * ldd;
 #pragma unroll
@@ -213,65 +243,184 @@ exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, c
 }
 
 // ---- digit planes ----
+// The 48 bits v 2^48, v = x 2^-e, |v| < 1/2, are rounded once and cut into bytes with integer
+// operations, 128 added to each so that the bytes are the digits plus 128 (GB300's FP64 pipe runs at
+// 1/64 of the integer rate; in FP64 the digits of 16 columns of 7680 took 48 us, and now 7).
+constexpr unsigned long long DIGIT_BIAS = 0x808080808080ull;
+constexpr int NOT_FINITE = INT_MIN;  // exponent of a column with an infinity or a NaN: its products are NaN
+
+// m 2^-s rounded to an integer
+__device__ __forceinline__ unsigned long long shift_round(unsigned long long m, int s) {
+  if (s <= 0) return m << -s;
+  return s > 62 ? 0ull : (m + (1ull << (s - 1))) >> s;
+}
+// x 2^(b - e) rounded, for |x| < 2^(e - 1) and b <= 60
+__device__ __forceinline__ long long fixed_f64(double x, int e, int b) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((u >> 52) & 2047);
+  const unsigned long long m = (u & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
+  const long long v = (long long)shift_round(m, 1075 - b + e - max(ex, 1));
+  return (u >> 63) ? -v : v;
+}
+__device__ __forceinline__ long long fixed_f32(float x, int e, int b) {
+  const uint32_t u = __float_as_uint(x);
+  const int ex = (int)((u >> 23) & 255);
+  const unsigned long long m = (u & 0x7fffffu) | (ex ? 1u << 23 : 0u);
+  const long long v = (long long)shift_round(m, 150 - b + e - max(ex, 1));
+  return (u >> 31) ? -v : v;
+}
+
+// rows of an operand: mag() is the size of an entry by its bits, fixed() its 48 bits under 2^e
 struct SrcC64Stacked {  // rows 0..n-1: Re of the complex64 matrix rows, rows n..2n-1: Im
   const float2* M;
   long long ld;
   int n;
-  __device__ double operator()(int r, int k) const {
-    return r < n ? (double)M[(size_t)r * ld + k].x : (double)M[(size_t)(r - n) * ld + k].y;
-  }
+  __device__ float at(int r, int k) const { return r < n ? M[(size_t)r * ld + k].x : M[(size_t)(r - n) * ld + k].y; }
+  __device__ uint32_t mag(int r, int k) const { return __float_as_uint(at(r, k)) & 0x7fffffffu; }
+  __device__ long long fixed(int r, int k, int e) const { return fixed_f32(at(r, k), e, 48); }
 };
-struct SrcF32Pair {  // hi + lo FP32 planes of an FP64-accurate real matrix
+struct SrcF32Pair {  // hi + lo FP32 planes of an FP64-accurate real matrix (hi the sum rounded to FP32)
   const float* hi;
   const float* lo;
   long long ld;
-  __device__ double operator()(int r, int k) const {
+  __device__ uint32_t mag(int r, int k) const { return __float_as_uint(hi[(size_t)r * ld + k]) & 0x7fffffffu; }
+  __device__ long long fixed(int r, int k, int e) const {
     const size_t o = (size_t)r * ld + k;
-    return (double)hi[o] + (double)lo[o];
-  }
-};
-struct SrcXStacked {  // rows 0..nr-1: Re of the columns of X (n x nr, column-major), rows nr..: Im
-  const double2* X;
-  int n, nr;
-  __device__ double operator()(int r, int k) const {
-    return r < nr ? X[(size_t)r * n + k].x : X[(size_t)(r - nr) * n + k].y;
+    return (fixed_f32(hi[o], e, 60) + fixed_f32(lo[o], e, 60) + 2048) >> 12;
   }
 };
 
 constexpr int DT = 256;
 
-// One CTA per row: the row's power-of-two scale 2^e (|v| 2^-e <= 1/2) and its XS base-256
-// digits, by repeated rounding of the scaled value, written to XS planes (zeros in the padding).
+// the digits of two consecutive k into XS planes (32-bit words p of a row)
+__device__ __forceinline__ void store_digits(long long u, long long v, uint32_t* __restrict__ o, size_t plane) {
+  const unsigned long long wu = (unsigned long long)u + DIGIT_BIAS, wv = (unsigned long long)v + DIGIT_BIAS;
+#pragma unroll
+  for (int s = 0; s < XS; ++s) {
+    const int sh = 40 - 8 * s;
+    const uint32_t mask = s ? 255u : 511u;  // the leading digit runs to 128
+    const __nv_bfloat162 d = __floats2bfloat162_rn((float)((int)((uint32_t)(wu >> sh) & mask) - 128),
+                                                   (float)((int)((uint32_t)(wv >> sh) & mask) - 128));
+    o[s * plane] = *reinterpret_cast<const uint32_t*>(&d);
+  }
+}
+
+// One CTA per row of a matrix: the row's power-of-two scale 2^e (|v| 2^-e < 1/2) and its XS base-256
+// digits, written to XS planes (zeros in the padding).
 template <class Src>
-__global__ void __launch_bounds__(DT) digits_kernel(Src src, int K, long long ldp, __nv_bfloat16* __restrict__ planes,
+__global__ void __launch_bounds__(DT) digits_kernel(Src src, int K, long long ldp, uint32_t* __restrict__ planes,
                                                     long long plane_stride, int* __restrict__ e_out) {
   RF_COUNT_LAUNCH();
   const int r = blockIdx.x;
-  double m = 0.0;
-  for (int k = threadIdx.x; k < K; k += DT) m = fmax(m, fabs(src(r, k)));
-  for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, off));
-  __shared__ double red[DT / 32];
-  __shared__ int e_sh;
+  uint32_t m = 0;
+  for (int k = threadIdx.x; k < K; k += DT) m = max(m, src.mag(r, k));
+  m = __reduce_max_sync(0xffffffffu, m);
+  __shared__ uint32_t red[DT / 32];
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < DT / 32; ++w) t = fmax(t, red[w]);
-    const int e = t > 0.0 ? ilogb(t) + 2 : 0;  // t < 2^(ilogb(t) + 1) = 2^(e - 1)
-    e_sh = e;
-    e_out[r] = e;
+#pragma unroll
+  for (int w = 0; w < DT / 32; ++w) m = max(m, red[w]);
+  const int e = m ? ilogbf(__uint_as_float(m)) + 2 : 0;  // |v| < 2^(e - 1)
+  if (threadIdx.x == 0) e_out[r] = e;
+  const size_t plane = (size_t)plane_stride / 2;
+  for (int p = threadIdx.x; p < (int)(ldp / 2); p += DT) {
+    const int k = 2 * p;
+    store_digits(k < K ? src.fixed(r, k, e) : 0, k + 1 < K ? src.fixed(r, k + 1, e) : 0,
+                 planes + (size_t)r * (ldp / 2) + p, plane);
+  }
+}
+
+// Re and Im of one column of X per cluster of XCL CTAs: each takes a slice of K, the column maxima
+// meet through distributed shared memory, then every slice writes its digits.  Rows 0..nr-1 of the
+// planes are Re of the columns, rows nr..2nr-1 Im.
+constexpr int XCL = 8;
+__global__ void __cluster_dims__(XCL, 1, 1) __launch_bounds__(DT)
+x_digits_kernel(const double2* __restrict__ X, int n, int nr, long long ldp, uint32_t* __restrict__ planes,
+                int* __restrict__ e_out) {
+  RF_COUNT_LAUNCH();
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ unsigned long long mx[2];
+  const int r = blockIdx.y, rank = (int)cl.block_rank();
+  const double2* x = X + (size_t)r * n;
+  const int pairs = (int)(ldp / 2), p0 = (int)((long long)pairs * rank / XCL), p1 = (int)((long long)pairs * (rank + 1) / XCL);
+  if (threadIdx.x < 2) mx[threadIdx.x] = 0;
+  __syncthreads();
+  unsigned long long a = 0, b = 0;
+  for (int k = 2 * p0 + threadIdx.x; k < min(2 * p1, n); k += DT) {
+    const double2 v = x[k];
+    a = max(a, (unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull);
+    b = max(b, (unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
+    b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&mx[0], a);
+    atomicMax(&mx[1], b);
+  }
+  cl.sync();
+  int e[2];
+#pragma unroll
+  for (int z = 0; z < 2; ++z) {
+    unsigned long long m = 0;
+    for (int c = 0; c < XCL; ++c) m = max(m, *cl.map_shared_rank(&mx[z], c));
+    e[z] = m == 0 ? 0 : (m >> 52) == 2047 ? NOT_FINITE : ilogb(__longlong_as_double((long long)m)) + 2;
+    if (rank == 0 && threadIdx.x == 0) e_out[z * nr + r] = e[z];
+  }
+  cl.sync();  // the other CTAs have read this one's maxima
+  const size_t plane = (size_t)nr * ldp;  // 32-bit words of one digit plane (2 nr rows of ldp / 2)
+  for (int p = p0 + threadIdx.x; p < p1; p += DT) {
+    const double2 zero = make_double2(0.0, 0.0);
+    const double2 u = 2 * p < n ? x[2 * p] : zero, v = 2 * p + 1 < n ? x[2 * p + 1] : zero;
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      const bool fin = e[z] != NOT_FINITE;
+      store_digits(fin ? fixed_f64(z ? u.y : u.x, e[z], 48) : 0, fin ? fixed_f64(z ? v.y : v.x, e[z], 48) : 0,
+                   planes + ((size_t)z * nr + r) * (ldp / 2) + p, plane);
+    }
+  }
+}
+
+// Y[:, r] = scale * op(T) X[:, r] (+ Y) from the integer sums of [Tr; Ti] [Xr Xi] or (real) P [Xr Xi],
+// at most XI_COLS columns: a CTA reads 32 rows of D along their columns and writes Y along its rows
+constexpr int XI_COLS = 32;
+__global__ void __launch_bounds__(DT)
+combine_int_kernel(const longlong2* __restrict__ D, const int* __restrict__ ea, const int* __restrict__ eb, int n,
+                   int nr, int conj, int real, double2 scale, int accumulate, double2* __restrict__ Y) {
+  RF_COUNT_LAUNCH();
+  __shared__ double2 t[XI_COLS][33];
+  const int i0 = blockIdx.x * 32;
+  auto value = [&](int row, int col) {
+    const longlong2 d = D[(size_t)row * (2 * nr) + col];
+    const int x = eb[col];
+    if (x == NOT_FINITE) return __longlong_as_double(0x7ff8000000000000ll);
+    const int e = ea[row] + x;
+    return ldexp((double)d.x, e - 32) + ldexp((double)d.y, e - 56);
+  };
+  const double sg = conj ? -1.0 : 1.0;
+  for (int q = threadIdx.x; q < 32 * nr; q += DT) {
+    const int i = i0 + q / nr, r = q % nr;
+    if (i >= n) break;
+    double2 v = make_double2(value(i, r), value(i, nr + r));
+    if (!real) {
+      v.x -= sg * value(n + i, nr + r);
+      v.y += sg * value(n + i, r);
+    }
+    t[r][i - i0] = make_double2(scale.x * v.x - scale.y * v.y, scale.x * v.y + scale.y * v.x);
   }
   __syncthreads();
-  const int e = e_sh;
-  for (long long k = threadIdx.x; k < ldp; k += DT) {
-    double u = k < K ? ldexp(src(r, (int)k), -e) : 0.0;
-#pragma unroll
-    for (int s = 0; s < XS; ++s) {
-      const double t = u * 256.0;
-      const double d = rint(t);
-      u = t - d;
-      planes[s * plane_stride + (size_t)r * ldp + k] = __double2bfloat16(d);
+  for (int q = threadIdx.x; q < 32 * nr; q += DT) {
+    const int r = q >> 5, i = i0 + (q & 31);
+    if (i >= n) continue;
+    double2 o = t[r][q & 31];
+    double2* y = Y + (size_t)r * n + i;
+    if (accumulate) {
+      o.x += y->x;
+      o.y += y->y;
     }
+    *y = o;
   }
 }
 
@@ -315,8 +464,25 @@ __global__ void combine_f64_kernel(const double* __restrict__ D, long long ldd, 
   }
 }
 
-cudaError_t exact_gemm(const ExactOperand& A, const ExactOperand& B, int M, int N, int K, double* D, long long ldd,
-                       int* err, cudaStream_t s) {
+// K split of a launch of `tiles` tiles of nkb K-blocks: the least of (waves of the chip) x (K-blocks of
+// a CTA + about two for its start and its integer sums); the smaller split where two are within 3 %
+int exact_split(long long tiles, int nkb, int sms) {
+  int best = 1;
+  double cost = 1e300;
+  for (int sp = 1; sp <= 16 && sp <= nkb; ++sp) {
+    const double waves = (double)((tiles * sp + sms - 1) / sms);
+    const double c = waves * ((nkb + sp - 1) / sp + (sp > 1 ? 2.5 : 1.5));
+    if (c < 0.97 * cost) {
+      cost = c;
+      best = sp;
+    }
+  }
+  return best;
+}
+
+// D = A B^T: FP64 values, or with DI the unscaled integer sums
+cudaError_t exact_gemm(const ExactOperand& A, const ExactOperand& B, int M, int N, int K, double* D, longlong2* DI,
+                       long long ldd, int* err, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0 || A.rows < M || B.rows < N) return cudaErrorInvalidValue;
   ExactMaps maps;
   std::memset(&maps, 0, sizeof(maps));
@@ -326,13 +492,49 @@ cudaError_t exact_gemm(const ExactOperand& A, const ExactOperand& B, int M, int 
       return cudaErrorInvalidValue;
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
+  static int sms = 0;
   std::call_once(once, [] {
     attr = cudaFuncSetAttribute(exact_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, XSMEM);
+    int dev = 0;
+    if (attr == cudaSuccess) attr = cudaGetDevice(&dev);
+    if (attr == cudaSuccess) attr = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   });
   if (attr != cudaSuccess) return attr;
-  const dim3 grid((N + XBN - 1) / XBN, (M + BM - 1) / BM);
+  const int tn = (N + XBN - 1) / XBN, tm = (M + BM - 1) / BM, nkb = (K + XKB - 1) / XKB;
+  const int split = DI ? exact_split((long long)tn * tm, nkb, std::max(sms, 1)) : 1;
+  if (split > 1) {
+    const cudaError_t e = cudaMemsetAsync(DI, 0, sizeof(longlong2) * (size_t)M * ldd, s);
+    if (e != cudaSuccess) return e;
+  }
   ProfScope prof("gemm_exact", 0.0, 2.0 * (XS * (XS + 1) / 2) * (double)M * N * K, s);
-  exact_gemm_kernel<<<grid, XTHREADS, XSMEM, s>>>(maps, M, N, K, A.e, B.e, D, ldd, err);
+  exact_gemm_kernel<<<dim3(tn, tm, split), XTHREADS, XSMEM, s>>>(maps, M, N, K, A.e, B.e, D, DI, ldd, err);
+  return cudaGetLastError();
+}
+
+// Y = scale * op(T) X (+ Y) (complex T as 2n stacked rows, or real)
+cudaError_t exact_product(const ExactOperand& T, int n, const double2* X, double2* Y, int nr, bool conj, bool real,
+                          double2 scale, bool accumulate, MrhsScratch& w, cudaStream_t s) {
+  const int rows = real ? n : 2 * n;
+  if (nr > w.cap_cols || n > w.cap_n || T.ldp > w.cap_ld || !w.xd || T.rows < rows) return cudaErrorInvalidValue;
+  ExactOperand B;
+  B.d = w.xd;
+  B.e = w.xe;
+  B.rows = 2 * nr;
+  B.ldp = T.ldp;
+  B.plane_stride = (long long)2 * nr * T.ldp;
+  x_digits_kernel<<<dim3(XCL, nr), DT, 0, s>>>(X, n, nr, B.ldp, reinterpret_cast<uint32_t*>(B.d), B.e);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const bool ints = nr <= XI_COLS;
+  longlong2* DI = ints ? reinterpret_cast<longlong2*>(w.D64) : nullptr;
+  if ((e = exact_gemm(T, B, rows, 2 * nr, n, w.D64, DI, 2 * nr, w.err, s)) != cudaSuccess) return e;
+  if (ints) {
+    combine_int_kernel<<<(n + 31) / 32, DT, 0, s>>>(DI, T.e, B.e, n, nr, conj ? 1 : 0, real ? 1 : 0, scale,
+                                                   accumulate ? 1 : 0, Y);
+  } else {
+    const dim3 g((n + CT - 1) / CT, (nr + CT - 1) / CT), b(CT, 8);
+    combine_f64_kernel<<<g, b, 0, s>>>(w.D64, 2 * nr, n, nr, conj ? 1 : 0, real ? 1 : 0, scale, accumulate ? 1 : 0, Y);
+  }
   return cudaGetLastError();
 }
 
@@ -341,7 +543,7 @@ cudaError_t exact_gemm(const ExactOperand& A, const ExactOperand& B, int M, int 
 cudaError_t exact_digits_c64(const float2* M, int n, long long ld, const ExactOperand& out, cudaStream_t s) {
   if (out.rows < 2 * n || out.ldp < ld) return cudaErrorInvalidValue;
   SrcC64Stacked src{M, ld, n};
-  digits_kernel<<<2 * n, DT, 0, s>>>(src, n, out.ldp, out.d, out.plane_stride, out.e);
+  digits_kernel<<<2 * n, DT, 0, s>>>(src, n, out.ldp, reinterpret_cast<uint32_t*>(out.d), out.plane_stride, out.e);
   return cudaGetLastError();
 }
 
@@ -349,45 +551,21 @@ cudaError_t exact_digits_f32pair(const float* hi, const float* lo, int n, long l
                                  cudaStream_t s) {
   if (out.rows < n || out.ldp < ld) return cudaErrorInvalidValue;
   SrcF32Pair src{hi, lo, ld};
-  digits_kernel<<<n, DT, 0, s>>>(src, n, out.ldp, out.d, out.plane_stride, out.e);
+  digits_kernel<<<n, DT, 0, s>>>(src, n, out.ldp, reinterpret_cast<uint32_t*>(out.d), out.plane_stride, out.e);
   return cudaGetLastError();
 }
 
 cudaError_t exact_cplx_gemm(const ExactOperand& T, int n, const double2* X, double2* Y, int nr, bool conj,
                             double2 scale, bool accumulate, MrhsScratch& w, cudaStream_t s) {
-  if (nr > w.cap_cols || n > w.cap_n || T.ldp > w.cap_ld || !w.xd || T.rows < 2 * n) return cudaErrorInvalidValue;
-  ExactOperand B;
-  B.d = w.xd;
-  B.e = w.xe;
-  B.rows = 2 * nr;
-  B.ldp = T.ldp;
-  B.plane_stride = (long long)2 * nr * T.ldp;
-  SrcXStacked src{X, n, nr};
-  digits_kernel<<<2 * nr, DT, 0, s>>>(src, n, B.ldp, B.d, B.plane_stride, B.e);
-  cudaError_t e;
-  if ((e = exact_gemm(T, B, 2 * n, 2 * nr, n, w.D64, 2 * nr, w.err, s)) != cudaSuccess) return e;
-  const dim3 g((n + CT - 1) / CT, (nr + CT - 1) / CT), b(CT, 8);
-  combine_f64_kernel<<<g, b, 0, s>>>(w.D64, 2 * nr, n, nr, conj ? 1 : 0, 0, scale, accumulate ? 1 : 0, Y);
-  return cudaGetLastError();
+  return exact_product(T, n, X, Y, nr, conj, false, scale, accumulate, w, s);
 }
 
 cudaError_t exact_real_gemm(const ExactOperand& P, int n, const double2* X, double2* Y, int nr, double scale,
                             bool accumulate, MrhsScratch& w, cudaStream_t s) {
-  if (nr > w.cap_cols || n > w.cap_n || P.ldp > w.cap_ld || !w.xd || P.rows < n) return cudaErrorInvalidValue;
-  ExactOperand B;
-  B.d = w.xd;
-  B.e = w.xe;
-  B.rows = 2 * nr;
-  B.ldp = P.ldp;
-  B.plane_stride = (long long)2 * nr * P.ldp;
-  SrcXStacked src{X, n, nr};
-  digits_kernel<<<2 * nr, DT, 0, s>>>(src, n, B.ldp, B.d, B.plane_stride, B.e);
-  cudaError_t e;
-  if ((e = exact_gemm(P, B, n, 2 * nr, n, w.D64, 2 * nr, w.err, s)) != cudaSuccess) return e;
-  const dim3 g((n + CT - 1) / CT, (nr + CT - 1) / CT), b(CT, 8);
-  combine_f64_kernel<<<g, b, 0, s>>>(w.D64, 2 * nr, n, nr, 0, 1, make_double2(scale, 0.0), accumulate ? 1 : 0, Y);
-  return cudaGetLastError();
+  return exact_product(P, n, X, Y, nr, false, true, make_double2(scale, 0.0), accumulate, w, s);
 }
+
+size_t exact_result_doubles(int cols) { return (size_t)std::max(4 * cols, 8 * std::min(cols, XI_COLS)); }
 
 RF_LAUNCH_READER(launches_exact)
 

@@ -227,7 +227,7 @@ struct MrhsScratch {
   // exact-digit products (float-float accurate multi-column products)
   __nv_bfloat16* xd = nullptr;  // EXACT_DIGITS planes of 2 cap_cols x cap_ld
   int* xe = nullptr;            // 2 cap_cols row exponents
-  double* D64 = nullptr;        // 4 x cap_cols x cap_n
+  double* D64 = nullptr;        // exact_result_doubles(cap_cols) x cap_n
 };
 
 // Exact-digit operands: every row r scaled by 2^e[r] and written as EXACT_DIGITS signed 8-bit
@@ -251,6 +251,8 @@ cudaError_t exact_cplx_gemm(const ExactOperand& T, int n, const double2* X, doub
                             double2 scale, bool accumulate, MrhsScratch& w, cudaStream_t s);
 cudaError_t exact_real_gemm(const ExactOperand& P, int n, const double2* X, double2* Y, int nr, double scale,
                             bool accumulate, MrhsScratch& w, cudaStream_t s);
+// doubles per row of MrhsScratch::D64 for products of up to cols columns
+size_t exact_result_doubles(int cols);
 cudaError_t split_c64_planes(const float2* M, int n, long long ld, const CplxPlanes& P, cudaStream_t s);
 // Y = scale * op(T) X (+ Y) with op = conj if conj; X, Y complex128 column-major n x nr.
 cudaError_t cplx_gemm(const CplxPlanes& T, const double2* X, double2* Y, int nr, bool conj, double2 scale,
