@@ -55,14 +55,6 @@ __device__ __forceinline__ void sincos_quarter(float r, float* s, float* c) {
   *c = fmaf(r2, pc, 1.0f);
 }
 
-// sin and cos of |r| <= 1/20 in FP32: sin to r^3 (truncation r^4/120 <= 6e-8 relative, the FP32
-// rounding) and cos to r^4 (below 3e-11)
-__device__ __forceinline__ void sincos_twentieth(float r, float* s, float* c) {
-  const float r2 = r * r;
-  *s = fmaf(r * r2, -1.0f / 6.0f, r);
-  *c = fmaf(r2, fmaf(r2, 1.0f / 24.0f, -0.5f), 1.0f);
-}
-
 // sin and cos of x >= 0 in FP32.  Cody and Waite's reduction (1980): q = nearest integer to
 // x 2/pi, r = x - q pi/2 with pi/2 split into a short leading part (q times it is exact for
 // q < 2^16) and a remainder; then the series above on |r| <= pi/4 and the quadrant of q.
@@ -642,20 +634,23 @@ __global__ void rhs_kernel(const DeviceGeometry g, double k, const double* __res
 // ---------------------------------------------------------------- radiation vector (FP64)
 // F(u) = sum_cells sum_q w_q e^{-ik u.r_q} J_c(r_q) over the 7-point rule, with the cell current
 // J_c(r) = sum_i s_i j_i (r - P_i) / 2 (the RWG functions of Eq. RWGdef times the cell area of
-// the product rule) = (r S - T) / 2, S = sum_i s_i j_i, T = sum_i s_i j_i P_i.  Hence
-//   F_c = (S B1 - T B0) / 2,  B0 = sum_q w_q e^{-ik u.r_q},  B1 = sum_q w_q e^{-ik u.r_q} r_q,
-// where B0 and B1 depend on the direction and the cell only (one set for RB right-hand sides),
-// and e^{-ik u.r_q} = e^{-ik u.c} e^{-ik u.(r_q - c)} (c the centroid) takes one sincos per cell
-// and, per point, the Taylor series of a small angle.  Everything stays FP64: at low frequency
-// the radiated field is a small remainder of the cell contributions.
-constexpr int FF_THREADS = 256;
-
-// cos and sin of |x| <= 1/20 by their Taylor series (to x^6 and x^7: truncation below 1e-15)
-__device__ __forceinline__ void sincos_tiny64(double x, double* s, double* c) {
-  const double x2 = x * x;
-  *c = fma(x2, fma(x2, fma(x2, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
-  *s = fma(x * x2, fma(x2, fma(x2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0), x);
-}
+// the product rule).  About the centroid c, with rho = r - c and v_i = P_i - c,
+//   F_c = e^{-ik u.c} (S B1 - T B0) / 2,  S = sum_i s_i j_i,  T = sum_i s_i j_i v_i,
+//   B0 = sum_q w_q e^{-ik u.rho_q},  B1 = sum_q w_q e^{-ik u.rho_q} rho_q.
+// The rule's points are the centroid and, on each vertex direction, rho = al v_i and rho = be v_i (al = 1
+// - 3a, be = 1 - 3b of its barycentric coordinates), and v_0 + v_1 + v_2 = 0, so B0 and B1 are sums over
+// i of four even or odd functions of the one angle x_i = -k u.v_i; where |x| is small each is one
+// polynomial.  B0 and B1 depend on the direction and the cell only (one set for RB right-hand sides).
+// Everything stays FP64: at low frequency the radiated field is a small remainder of the cell
+// contributions.
+//
+// Bound: the FP64 pipe (1/64 of the FP32 rate), 114 operations per (direction, cell) and 24 per
+// right-hand side after that.  farfield_cells_kernel forms S / (-k), T and -k v once per call; the
+// direction kernel used to gather them per direction and took 21 dot products and 42 operations for B1.
+// GB300: 362 directions of one current on 20480 cells 5.10 -> 1.98 ms (the FP64 floor of 138 operations
+// is 1.63 ms); 91 directions of 23 currents on 1600 cells 1.11 -> 0.46 ms.
+constexpr int FF_THREADS = 128;
+constexpr int FF_COLS = 64;  // right-hand sides of one pass (bounds the cell currents' scratch)
 
 // cos and sin of |x| <= 1/2 by their Taylor series (to x^12 and x^13: truncation below 1e-15)
 __device__ __forceinline__ void sincos_small64(double x, double* s, double* c) {
@@ -674,47 +669,143 @@ __device__ __forceinline__ void sincos_small64(double x, double* s, double* c) {
   *s = fma(x * x2, ps, x);
 }
 
+// geo (9 x nc): -k v_0, -k v_1, -k c; cur (8 nrhs x nc): Re and Im of S / (-k) and of T's components
+__global__ void farfield_cells_kernel(const DeviceGeometry g, double k, const double2* __restrict__ j, int nrhs,
+                                      double* __restrict__ geo, double* __restrict__ cur) {
+  RF_COUNT_LAUNCH();
+  const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+  if (c >= g.nc) return;
+  double v[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int e = 0; e < 3; ++e) v[i][e] = g.verts[3 * g.tris[3 * c + i] + e] - g.cen64[3 * c + e];
+  if (r == 0) {
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      geo[(size_t)e * g.nc + c] = -k * v[0][e];
+      geo[(size_t)(3 + e) * g.nc + c] = -k * v[1][e];
+      geo[(size_t)(6 + e) * g.nc + c] = -k * g.cen64[3 * c + e];
+    }
+  }
+  double sr = 0.0, si = 0.0, tr[3] = {0.0, 0.0, 0.0}, ti[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int ed = g.cell_edges[3 * c + i];
+    if (ed < 0) continue;  // a boundary edge: no current
+    const double sg = (double)g.cell_sign[3 * c + i];
+    const double2 x = j[(size_t)r * g.ne + ed];
+    const double vr = sg * x.x, vi = sg * x.y;
+    sr += vr;
+    si += vi;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      tr[e] = fma(vr, v[i][e], tr[e]);
+      ti[e] = fma(vi, v[i][e], ti[e]);
+    }
+  }
+  double* o = cur + (size_t)8 * r * g.nc + c;
+  o[0] = -sr / k;
+  o[(size_t)g.nc] = -si / k;
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    o[(size_t)(2 + 2 * e) * g.nc] = tr[e];
+    o[(size_t)(3 + 2 * e) * g.nc] = ti[e];
+  }
+}
+
+// weights (times 1/2) and vertex factors of the rule, and the series of the four sums over one vertex
+// direction in y = x^2: cos of (weight, weight x factor) and sin / x of the same
+struct FarRule {
+  double w0, wa, wb, al, be;
+  double c0[4], s0[4], c1[4], s1[4];
+};
+__host__ __device__ constexpr FarRule far_rule() {
+  constexpr double s15 = 3.872983346207416885;
+  FarRule f{};
+  f.w0 = 0.5 * (9.0 / 40.0);
+  f.wa = 0.5 * (155.0 - s15) / 1200.0;
+  f.wb = 0.5 * (155.0 + s15) / 1200.0;
+  f.al = 1.0 - 3.0 * (6.0 - s15) / 21.0;
+  f.be = 1.0 - 3.0 * (6.0 + s15) / 21.0;
+  double pa = f.wa, pb = f.wb, fact = 1.0;  // w al^m, w be^m, m!
+  for (int m = 0; m < 4; ++m) {
+    const double sg = m % 2 ? -1.0 : 1.0;
+    f.c0[m] = sg * (pa + pb) / fact;                        // w z^2m / (2m)!
+    f.c1[m] = sg * (pa * f.al + pb * f.be) / fact;          // w z^(2m+1) / (2m)!
+    f.s0[m] = sg * (pa * f.al + pb * f.be) / (fact * (2 * m + 1));
+    f.s1[m] = sg * (pa * f.al * f.al + pb * f.be * f.be) / (fact * (2 * m + 1));
+    pa *= f.al * f.al;
+    pb *= f.be * f.be;
+    fact *= (2 * m + 1) * (2 * m + 2);
+  }
+  return f;
+}
+
+__device__ __forceinline__ void sincos_any64(double x, double* s, double* c) {
+  if (fabs(x) <= 0.5) sincos_small64(x, s, c);
+  else sincos(x, s, c);
+}
+
+// CTA (direction, group of RB right-hand sides, chunk of cells): partial radiation vectors
 template <int RB>
 __global__ void __launch_bounds__(FF_THREADS)
-farfield_kernel(const DeviceGeometry g, double k, const double2* __restrict__ j, int nrhs, const double* dirs,
-                int ndir, double2* __restrict__ out) {
+farfield_kernel(int nc, const double* __restrict__ geo, const double* __restrict__ cur, int nrhs,
+                const double* __restrict__ dirs, int ndir, int blocks_per_chunk, double* __restrict__ part) {
   RF_COUNT_LAUNCH();
-  const int d = blockIdx.x;
-  const int r0 = blockIdx.y * RB;
+  constexpr FarRule R = far_rule();
+  constexpr int V = RB == 1 ? 8 : (RB == 4 ? 32 : 64);
+  const int d = blockIdx.x, r0 = blockIdx.y * RB;
   const double ux = dirs[3 * d], uy = dirs[3 * d + 1], uz = dirs[3 * d + 2];
-  // 7-point rule weights (sum 1) times 1/2
-  const double wa = 0.5 * (9.0 / 40.0), wb = 0.5 * (155.0 - 3.872983346207416885) / 1200.0,
-               wc = 0.5 * (155.0 + 3.872983346207416885) / 1200.0;
-  double acc[RB][6];
+  double acc[V];
 #pragma unroll
-  for (int b = 0; b < RB; ++b)
+  for (int q = 0; q < V; ++q) acc[q] = 0.0;
+  const int c0 = blockIdx.z * blocks_per_chunk * FF_THREADS, c1 = min(nc, c0 + blocks_per_chunk * FF_THREADS);
+  for (int c = c0 + threadIdx.x; c < c1; c += FF_THREADS) {
+    double v[3][3], x[3];
 #pragma unroll
-    for (int e = 0; e < 6; ++e) acc[b][e] = 0.0;
-  for (int c = threadIdx.x; c < g.nc; c += blockDim.x) {
-    const double cx = g.cen64[3 * c], cy = g.cen64[3 * c + 1], cz = g.cen64[3 * c + 2];
-    double b0r = 0.0, b0i = 0.0, b1r[3] = {0.0, 0.0, 0.0}, b1i[3] = {0.0, 0.0, 0.0};
+    for (int e = 0; e < 3; ++e) {
+      v[0][e] = geo[(size_t)e * nc + c];
+      v[1][e] = geo[(size_t)(3 + e) * nc + c];
+    }
+    x[0] = fma(ux, v[0][0], fma(uy, v[0][1], uz * v[0][2]));
+    x[1] = fma(ux, v[1][0], fma(uy, v[1][1], uz * v[1][2]));
+    x[2] = -(x[0] + x[1]);
+    double b0r = R.w0, b0i = 0.0, g1r[3], g1i[3];
+    if (fmax(fabs(x[0]), fmax(fabs(x[1]), fabs(x[2]))) <= 0.07) {  // al |x| <= 1/20: truncation below 1e-15
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
-      const double* rq = g.qp64 + 21 * c + 3 * q;
-      const double x = -k * (ux * (rq[0] - cx) + uy * (rq[1] - cy) + uz * (rq[2] - cz));
-      double sn, cs;
-      const double ax = fabs(x);
-      if (ax <= 0.05) sincos_tiny64(x, &sn, &cs);
-      else if (ax <= 0.5) sincos_small64(x, &sn, &cs);
-      else sincos(x, &sn, &cs);
-      const double w = q == 0 ? wa : (q < 4 ? wb : wc);
-      const double er = w * cs, ei = w * sn;
-      b0r += er;
-      b0i += ei;
+      for (int i = 0; i < 3; ++i) {
+        const double y = x[i] * x[i];
+        b0r += fma(y, fma(y, fma(y, R.c0[3], R.c0[2]), R.c0[1]), R.c0[0]);
+        b0i = fma(x[i], fma(y, fma(y, fma(y, R.s0[3], R.s0[2]), R.s0[1]), R.s0[0]), b0i);
+        g1r[i] = fma(y, fma(y, fma(y, R.c1[3], R.c1[2]), R.c1[1]), R.c1[0]);
+        g1i[i] = x[i] * fma(y, fma(y, fma(y, R.s1[3], R.s1[2]), R.s1[1]), R.s1[0]);
+      }
+    } else {
 #pragma unroll
-      for (int e = 0; e < 3; ++e) {
-        b1r[e] = fma(er, rq[e], b1r[e]);
-        b1i[e] = fma(ei, rq[e], b1i[e]);
+      for (int i = 0; i < 3; ++i) {
+        double sa, ca, sb, cb;
+        sincos_any64(R.al * x[i], &sa, &ca);
+        sincos_any64(R.be * x[i], &sb, &cb);
+        b0r = fma(R.wa, ca, fma(R.wb, cb, b0r));
+        b0i = fma(R.wa, sa, fma(R.wb, sb, b0i));
+        g1r[i] = fma(R.wa * R.al, ca, R.wb * R.be * cb);
+        g1i[i] = fma(R.wa * R.al, sa, R.wb * R.be * sb);
       }
     }
+    // B1 = sum_i v_i g_i with v_2 = -(v_0 + v_1)
+    double b1r[3], b1i[3];
+    const double h0r = g1r[0] - g1r[2], h0i = g1i[0] - g1i[2], h1r = g1r[1] - g1r[2], h1i = g1i[1] - g1i[2];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      b1r[e] = fma(v[0][e], h0r, v[1][e] * h1r);
+      b1i[e] = fma(v[0][e], h0i, v[1][e] * h1i);
+    }
     {  // times e^{-ik u.c}
+      const double ph = fma(ux, geo[(size_t)6 * nc + c], fma(uy, geo[(size_t)7 * nc + c], uz * geo[(size_t)8 * nc + c]));
       double sn, cs;
-      sincos(-k * (ux * cx + uy * cy + uz * cz), &sn, &cs);
+      if (__all_sync(__activemask(), fabs(ph) <= 0.5)) sincos_small64(ph, &sn, &cs);
+      else sincos(ph, &sn, &cs);
       double t = b0r;
       b0r = t * cs - b0i * sn;
       b0i = t * sn + b0i * cs;
@@ -725,58 +816,60 @@ farfield_kernel(const DeviceGeometry g, double k, const double2* __restrict__ j,
         b1i[e] = t * sn + b1i[e] * cs;
       }
     }
-    int ed[3];
-    double sg[3];
-    const double* P[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      ed[i] = g.cell_edges[3 * c + i];
-      sg[i] = (double)g.cell_sign[3 * c + i];
-      P[i] = g.verts + 3 * g.tris[3 * c + i];
-    }
 #pragma unroll
     for (int b = 0; b < RB; ++b) {
-      if (r0 + b >= nrhs) break;
-      const double2* jr = j + (size_t)(r0 + b) * g.ne;
-      double sr = 0.0, si = 0.0, tr[3] = {0.0, 0.0, 0.0}, ti[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        if (ed[i] < 0) continue;  // a boundary edge: no current
-        const double2 v = jr[ed[i]];
-        const double vr = sg[i] * v.x, vi = sg[i] * v.y;
-        sr += vr;
-        si += vi;
-#pragma unroll
-        for (int e = 0; e < 3; ++e) {
-          tr[e] = fma(vr, P[i][e], tr[e]);
-          ti[e] = fma(vi, P[i][e], ti[e]);
-        }
-      }
+      if (RB > 1 && r0 + b >= nrhs) break;
+      const double* q = cur + (size_t)8 * (r0 + b) * nc + c;
+      const double sr = q[0], si = q[(size_t)nc];
 #pragma unroll
       for (int e = 0; e < 3; ++e) {  // S B1 - T B0
-        acc[b][2 * e] += (sr * b1r[e] - si * b1i[e]) - (tr[e] * b0r - ti[e] * b0i);
-        acc[b][2 * e + 1] += (sr * b1i[e] + si * b1r[e]) - (tr[e] * b0i + ti[e] * b0r);
+        const double tr = q[(size_t)(2 + 2 * e) * nc], ti = q[(size_t)(3 + 2 * e) * nc];
+        acc[6 * b + 2 * e] = fma(sr, b1r[e], fma(-si, b1i[e], fma(-tr, b0r, fma(ti, b0i, acc[6 * b + 2 * e]))));
+        acc[6 * b + 2 * e + 1] = fma(sr, b1i[e], fma(si, b1r[e], fma(-tr, b0i, fma(-ti, b0r, acc[6 * b + 2 * e + 1]))));
       }
     }
   }
-  __shared__ double red[FF_THREADS / 32][6];
+  // sums over the warp by halves (a lane ends with V / 32 of them), then over the warps
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-  for (int b = 0; b < RB; ++b) {
-    if (r0 + b >= nrhs) break;
-    for (int e = 0; e < 6; ++e) {
-      double v = acc[b][e];
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][e] = v;
+  for (int step = 0; step < 5; ++step) {
+    const int off = 16 >> step, h = V >> (step + 1);
+    if (h == 0) {
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], off);
+    } else {
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int q = 0; q < h; ++q) {
+        const double send = up ? acc[q] : acc[q + h], keep = up ? acc[q + h] : acc[q];
+        acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+      }
     }
-    __syncthreads();
-    if (threadIdx.x < 6) {
-      double v = 0.0;
-      for (int w = 0; w < FF_THREADS / 32; ++w) v += red[w][threadIdx.x];
-      double* o = reinterpret_cast<double*>(out + ((size_t)(r0 + b) * ndir + d) * 3);
-      o[threadIdx.x] = v;
-    }
-    __syncthreads();
   }
+  __shared__ double red[FF_THREADS / 32][V];
+  if (V >= 32) {
+#pragma unroll
+    for (int q = 0; q < (V < 32 ? 1 : V / 32); ++q) red[w][lane * (V / 32) + q] = acc[q];
+  } else if (lane % (V < 32 ? 32 / V : 1) == 0) {
+    red[w][lane * V / 32] = acc[0];
+  }
+  __syncthreads();
+  const int q = threadIdx.x;
+  if (q < 6 * RB && r0 + q / 6 < nrhs) {
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < FF_THREADS / 32; ++i) s += red[i][q];
+    part[(((size_t)blockIdx.z * nrhs + r0 + q / 6) * ndir + d) * 6 + q % 6] = s;
+  }
+}
+
+// out = sum over the chunks, in their order
+__global__ void farfield_sum_kernel(const double* __restrict__ part, int chunks, long long n, double* __restrict__ out) {
+  RF_COUNT_LAUNCH();
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double s = 0.0;
+  for (int c = 0; c < chunks; ++c) s += part[(size_t)c * n + i];
+  out[i] = s;
 }
 
 }  // namespace
@@ -851,12 +944,34 @@ cudaError_t launch_rhs_planewave(const DeviceGeometry& g, double k, const double
 cudaError_t launch_farfield(const DeviceGeometry& g, double k, const double2* j, int nrhs, const double* dirs,
                             int ndir, double2* out, cudaStream_t s) {
   ProfScope prof("farfield", 0.0, 0.0, s);
-  if (nrhs == 1) {
-    farfield_kernel<1><<<dim3(ndir, 1), FF_THREADS, 0, s>>>(g, k, j, nrhs, dirs, ndir, out);
-  } else {
-    farfield_kernel<4><<<dim3(ndir, (nrhs + 3) / 4), FF_THREADS, 0, s>>>(g, k, j, nrhs, dirs, ndir, out);
+  const int cols = nrhs < FF_COLS ? nrhs : FF_COLS;
+  // eight right-hand sides share B0 and B1 where there are that many (48 sums a thread); a chunk is as
+  // many blocks of 128 cells as leave twelve CTAs a SM, at least two so that the sums over the CTA
+  // (about a fifth of one block's work) stay small
+  const int rb = cols == 1 ? 1 : (cols <= 4 ? 4 : 8);
+  const long long groups = (cols + rb - 1) / rb, nb = (g.nc + FF_THREADS - 1) / FF_THREADS;
+  const long long per = (nb * groups * ndir) / (152 * 12);
+  const int bpc = (int)(per < 2 ? 2 : (per > nb ? nb : per));
+  const int chunks = (int)((nb + bpc - 1) / bpc);
+  double* buf = nullptr;
+  const size_t geo = (size_t)9 * g.nc, cur = (size_t)8 * cols * g.nc, part = (size_t)chunks * cols * ndir * 6;
+  cudaError_t e = cudaMallocAsync(&buf, sizeof(double) * (geo + cur + part), s);
+  if (e != cudaSuccess) return e;
+  double *pcur = buf + geo, *ppart = pcur + cur;
+  for (int r = 0; r < nrhs && e == cudaSuccess; r += cols) {
+    const int nr = nrhs - r < cols ? nrhs - r : cols;
+    farfield_cells_kernel<<<dim3((g.nc + 127) / 128, nr), 128, 0, s>>>(g, k, j + (size_t)r * g.ne, nr, buf, pcur);
+    const dim3 grid(ndir, (nr + rb - 1) / rb, chunks);
+    if (rb == 1) farfield_kernel<1><<<grid, FF_THREADS, 0, s>>>(g.nc, buf, pcur, nr, dirs, ndir, bpc, ppart);
+    else if (rb == 4) farfield_kernel<4><<<grid, FF_THREADS, 0, s>>>(g.nc, buf, pcur, nr, dirs, ndir, bpc, ppart);
+    else farfield_kernel<8><<<grid, FF_THREADS, 0, s>>>(g.nc, buf, pcur, nr, dirs, ndir, bpc, ppart);
+    const long long n = (long long)nr * ndir * 6;
+    farfield_sum_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(ppart, chunks, n,
+                                                                   reinterpret_cast<double*>(out + (size_t)r * ndir * 3));
+    e = cudaGetLastError();
   }
-  return cudaGetLastError();
+  const cudaError_t f = cudaFreeAsync(buf, s);
+  return e != cudaSuccess ? e : f;
 }
 
 RF_LAUNCH_READER(launches_assembly)
