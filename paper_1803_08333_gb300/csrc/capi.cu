@@ -1316,6 +1316,27 @@ int upload_geometry(const Topology& T, const std::vector<double>& verts, DeviceG
   return RFCMP_OK;
 }
 
+// The rows of a graph Laplacian (a diagonal entry of 1 to 3, -1 per neighbour, at most three) as three
+// neighbours, n where there is none, and the diagonal, 16 bits each; empty if the matrix is not one or has
+// more rows than 16 bits number
+std::vector<uint4> laplacian_rows(const std::vector<int32_t>& ptr, const std::vector<int32_t>& col,
+                                 const std::vector<double>& val, int n) {
+  if (n > 65534) return {};
+  std::vector<uint4> out((n + 1) / 2, make_uint4(n | (uint32_t)n << 16, n, n | (uint32_t)n << 16, n));
+  for (int i = 0; i < n; ++i) {
+    int nb[3] = {n, n, n}, k = 0, d = 0;
+    for (int q = ptr[i]; q < ptr[i + 1]; ++q) {
+      if (col[q] == i && d == 0 && (val[q] == 1.0 || val[q] == 2.0 || val[q] == 3.0)) d = (int)val[q];
+      else if (col[q] != i && val[q] == -1.0 && k < 3) nb[k++] = col[q];
+      else return {};
+    }
+    const uint32_t a = (uint32_t)nb[0] | (uint32_t)nb[1] << 16, b = (uint32_t)nb[2] | (uint32_t)d << 16;
+    if (i & 1) out[i / 2].z = a, out[i / 2].w = b;
+    else out[i / 2].x = a, out[i / 2].y = b;
+  }
+  return out;
+}
+
 // dense inverse of a sparse SPD matrix (CSR on the host), FP32 hi + lo planes
 int build_factor(const std::vector<int32_t>& ptr, const std::vector<int32_t>& col, const std::vector<double>& val,
                  int n, bool project, bool multigrid, double tol, std::shared_ptr<DenseFactor>& out,
@@ -1331,9 +1352,14 @@ int build_factor(const std::vector<int32_t>& ptr, const std::vector<int32_t>& co
   std::vector<void*> tmp;
   int32_t *dptr = nullptr, *dcol = nullptr;
   double* dval = nullptr;
+  uint4* dlap = nullptr;
   int rc = upload(&dptr, ptr, tmp);
   if (rc == RFCMP_OK) rc = upload(&dcol, col, tmp);
   if (rc == RFCMP_OK) rc = upload(&dval, val, tmp);
+  if (rc == RFCMP_OK && project) {
+    const std::vector<uint4> lap = laplacian_rows(ptr, col, val, n);
+    if (!lap.empty()) rc = upload(&dlap, lap, tmp);
+  }
   if (rc != RFCMP_OK) {
     for (void* p : tmp) dev_free(p);
     return rc;
@@ -1368,7 +1394,7 @@ int build_factor(const std::vector<int32_t>& ptr, const std::vector<int32_t>& co
       iters += it;
       int st = 0;
       if (err == cudaSuccess)
-        err = newton_schulz_pseudo_inverse(dptr, dcol, dval, n, true, Xd, padded_ld(n), NS_MAX_STEPS, target, f->hi,
+        err = newton_schulz_pseudo_inverse(dptr, dcol, dval, dlap, n, true, Xd, padded_ld(n), NS_MAX_STEPS, target, f->hi,
                                            f->lo, &st, &res, 0);
       steps += st;
     }
@@ -1395,7 +1421,7 @@ int build_factor(const std::vector<int32_t>& ptr, const std::vector<int32_t>& co
     double res = 1.0;
     if (err == cudaSuccess) err = jacobi_start(dptr, dcol, dval, n, jacobi_c, Xd, padded_ld(n), 0);
     if (err == cudaSuccess)
-      err = newton_schulz_pseudo_inverse(dptr, dcol, dval, n, false, Xd, padded_ld(n), NS_MAX_STEPS, target, f->hi,
+      err = newton_schulz_pseudo_inverse(dptr, dcol, dval, nullptr, n, false, Xd, padded_ld(n), NS_MAX_STEPS, target, f->hi,
                                          f->lo, &steps, &res, 0);
     if (Xd) dev_free(Xd);
     f->ns_steps = steps;

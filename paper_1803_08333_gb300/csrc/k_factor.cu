@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "rfcmp_internal.h"
@@ -66,6 +67,160 @@ ns_residual_kernel(const double* __restrict__ X, long long ldx, int n, const int
   if (threadIdx.x == 0) {
     float m = 0.f;
     for (int w = 0; w < NSR_THREADS / 32; ++w) m = fmaxf(m, wmax[w]);
+    atomicMax(maxbits, (unsigned long long)__double_as_longlong((double)m));
+  }
+}
+
+// ---- the same residual for the graph Laplacian (the projected case), in fixed point ----
+// L has the cell's neighbour count on its diagonal and -1 per neighbour (at most three), so a row of X M
+// is a sum of X entries: X is taken as integers of 2^(e - 60) (|X| < 2^(e - 1), e from the largest
+// diagonal entry, which bounds a positive definite matrix), the row is staged in shared memory, and the
+// sums and 1 / alpha - (X M)_ij are exact 64-bit integers; the integer rounding of an entry is 2^-8 of
+// FP64's at the top of the range.  The row's sum for the 1 1^T / n term and the BF16 split of X, which
+// the product after this reads, come out of the same pass (they took a pass over X each).  Bound: the
+// integer pipe (62 % busy) and DRAM, 16 bytes an entry (8 read, 4 + 4 written; 34 %); the FP64 form was
+// bound by the FP64 pipe.  8000 cells on GB300: 0.87 ms for the three passes, 0.36 ms in this one.
+// Rows longer than LAP_MAX do not fit shared memory and take the kernels around this one.
+constexpr int LAP_MAX = 28900;
+constexpr int FIX_BITS = 60;
+
+// x 2^(60 - e) rounded to an integer, |x| < 2^(e - 1): the mantissa with its leading bit at bit 60, shifted
+// right by the distance of x's exponent from the range's and one more; larger values and non-finite ones saturate
+__device__ __forceinline__ long long to_fixed(double x, int e) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const int ex = (int)((h >> 20) & 2047u), sh = e + 1022 - ex;  // >= 1 in range
+  uint32_t mh = (h & 0xfffffu) | 0x100000u, ml = l;
+  mh = __funnelshift_l(ml, mh, 8);
+  ml <<= 8;
+  if (sh > 62) mh = ml = 0;  // below the range's last bit (zeros and subnormals among them)
+  if (sh < 1) mh = 1u << 28, ml = 0;
+  const int s1 = min(max(sh, 0), 62);  // one place short: the last is rounded off
+  if (s1 >= 32) ml = mh, mh = 0;
+  ml = __funnelshift_r(ml, mh, s1 & 31);
+  mh >>= s1 & 31;
+  unsigned long long v = (((unsigned long long)mh << 32 | ml) + 1ull) >> 1;
+  if (sh < 1) v = 1ull << (FIX_BITS - 1);
+  return (int)h < 0 ? -(long long)v : (long long)v;
+}
+// x rounded to FP32 from its bits (halves away from zero), zero below FP32's normal range
+__device__ __forceinline__ float to_float(double x) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const uint32_t m = __funnelshift_l(l, h & 0x7fffffffu, 3) + 0x40000000u;  // exponent rebased by 896 (mod 2^9)
+  const uint32_t f = m + ((l >> 28) & 1u);
+  const uint32_t ex = h & 0x7ff00000u;
+  return ex < 0x38100000u ? 0.f : __uint_as_float((ex >= 0x47f00000u ? 0x7f800000u : f) | (h & 0x80000000u));
+}
+__device__ __forceinline__ uint32_t bf16_pair(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+// BF16 hi and lo planes of (a, b), at words p of the rows
+__device__ __forceinline__ void store_split(float a, float b, uint32_t* hi, uint32_t* lo, int p) {
+  const uint32_t h = bf16_pair(a, b);
+  hi[p] = h;
+  lo[p] = bf16_pair(a - __uint_as_float(h << 16), b - __uint_as_float(h & 0xffff0000u));
+}
+
+// largest diagonal entry of X, by its bits (out zeroed before)
+__global__ void diag_max_kernel(const double* __restrict__ X, long long ldx, int n, unsigned long long* __restrict__ out) {
+  RF_COUNT_LAUNCH();
+  unsigned long long m = 0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    m = max(m, (unsigned long long)__double_as_longlong(fabs(X[(size_t)i * ldx + i])));
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
+// CTA per row i: Rt[i][j] = delta_ij - alpha (X M)[i][j] and X's split, as BF16 hi/lo planes; max |Rt|.
+// nb: per two cells, each one's three neighbours (n where there is none) and its diagonal entry, 16 bits
+// each (an index list of int4 per cell took as much of the L1 as the rest of the kernel).
+__global__ void __launch_bounds__(1024, 1)
+ns_residual_lap_kernel(const double* __restrict__ X, long long ldx, int n, const uint4* __restrict__ nb,
+                       const unsigned long long* __restrict__ diag, double alpha, uint32_t* __restrict__ rhi,
+                       uint32_t* __restrict__ rlo, uint32_t* __restrict__ xhi, uint32_t* __restrict__ xlo,
+                       long long ldp, unsigned long long* __restrict__ maxbits) {
+  RF_COUNT_LAUNCH();
+  extern __shared__ __align__(16) long long row[];  // n + 1 entries, the last zero (n + 2 for an even n)
+  __shared__ long long red[2][32];
+  __shared__ long long mean;
+  __shared__ float wmax[32];
+  const int i = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int e = max(ilogb(__longlong_as_double((long long)*diag)), -2) + 2;
+  const float xs = __int_as_float((127 + e - FIX_BITS) << 23);  // 2^(e - 60); e <= 62 below any use of it
+  const size_t o = (size_t)i * (ldp / 2);
+  const int words = (n + 1) / 2;
+  long long sh = 0, sl = 0;  // the row's sum is sh 2^32 + sl, exactly
+  constexpr int B = 2;
+  const double2* xr = reinterpret_cast<const double2*>(X + (size_t)i * ldx);
+  for (int p0 = threadIdx.x; p0 < words; p0 += B * blockDim.x) {
+    double2 x[B];
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      const int p = p0 + u * blockDim.x;
+      x[u] = p < words ? xr[p] : make_double2(0.0, 0.0);
+    }
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      const int p = p0 + u * blockDim.x, j = 2 * p;
+      if (p >= words) break;
+      if (j + 1 >= n) x[u].y = 0.0;  // the padding of an odd row
+      const long long a = to_fixed(x[u].x, e), b = to_fixed(x[u].y, e);
+      *reinterpret_cast<longlong2*>(row + j) = make_longlong2(a, b);  // of an odd row: also its zero entry
+      sh += (a >> 32) + (b >> 32);
+      sl += (long long)(a & 0xffffffffll) + (long long)(b & 0xffffffffll);
+      store_split(to_float(x[u].x), to_float(x[u].y), xhi + o, xlo + o, p);
+    }
+  }
+  for (int k = 16; k > 0; k >>= 1) {
+    sh += __shfl_xor_sync(0xffffffffu, sh, k);
+    sl += __shfl_xor_sync(0xffffffffu, sl, k);
+  }
+  if (lane == 0) {
+    red[0][w] = sh;
+    red[1][w] = sl;
+  }
+  if (threadIdx.x == 0) row[n] = 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    sh = sl = 0;
+    for (int k = 0; k < nw; ++k) {
+      sh += red[0][k];
+      sl += red[1][k];
+    }
+    mean = __double2ll_rn(((double)sh * 4294967296.0 + (double)sl) / n);
+  }
+  __syncthreads();
+  const long long mu = mean, one = __double2ll_rn(ldexp(1.0 / alpha, FIX_BITS - e));
+  const float rs = (float)alpha * xs;
+  float mx = 0.f;
+  for (int p0 = threadIdx.x; p0 < words; p0 += B * blockDim.x) {
+    uint4 q[B];  // neighbours and diagonal of two cells, 16 bits each
+#pragma unroll
+    for (int u = 0; u < B; ++u) q[u] = nb[min(p0 + u * (int)blockDim.x, words - 1)];
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      const int p = p0 + u * blockDim.x;
+      if (p >= words) break;
+      const longlong2 own = *reinterpret_cast<const longlong2*>(row + 2 * p);
+      float r[2];
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        const int j = 2 * p + z;
+        const uint32_t c0 = z ? q[u].z : q[u].x, c1 = z ? q[u].w : q[u].y;
+        const long long a = (long long)(c1 >> 16) * (z ? own.y : own.x) - row[c0 & 0xffffu] - row[c0 >> 16] -
+                            row[c1 & 0xffffu] + mu;
+        r[z] = j < n ? rs * __ll2float_rn((i == j ? one : 0ll) - a) : 0.f;
+        mx = fmaxf(mx, fabsf(r[z]));
+      }
+      store_split(r[0], r[1], rhi + o, rlo + o, p);
+    }
+  }
+  for (int k = 16; k > 0; k >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, k));
+  if (lane == 0) wmax[w] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float m = 0.f;
+    for (int k = 0; k < nw; ++k) m = fmaxf(m, wmax[k]);
     atomicMax(maxbits, (unsigned long long)__double_as_longlong((double)m));
   }
 }
@@ -233,8 +388,8 @@ cudaError_t jacobi_start(const int32_t* ptr, const int32_t* col, const double* v
   return cudaGetLastError();
 }
 
-cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col, const double* val, int n,
-                                         bool project, double* X, long long ldx, int max_steps, double tol, float* Xhi,
+cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col, const double* val, const uint4* lap,
+                                         int n, bool project, double* X, long long ldx, int max_steps, double tol, float* Xhi,
                                          float* Xlo, int* steps_done, double* final_residual, cudaStream_t s) {
   // X holds an approximation of M^{-1} on entry (row-major, stride ldx): M = L + 1 1^T / n with
   // project (the result is M^{-1} - 1 1^T / n = L^+), M = L without
@@ -248,8 +403,19 @@ cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col,
   __nv_bfloat16 *xh, *xl, *rh, *rl;
   float* D;
   double* rowsum;
-  unsigned long long* maxbits;
+  unsigned long long* maxbits;  // max |R| and, for the fixed-point residual, the largest diagonal entry of X
   int* gerr;
+  const bool fixed = project && lap && n <= LAP_MAX;
+  const size_t lap_smem = ((size_t)n + 2) * sizeof(long long);
+  if (fixed) {
+    static std::once_flag once;
+    static cudaError_t attr = cudaSuccess;
+    std::call_once(once, [] {
+      attr = cudaFuncSetAttribute(ns_residual_lap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (LAP_MAX + 2) * (int)sizeof(long long));
+    });
+    if (attr != cudaSuccess) return attr;
+  }
   const size_t plane = (size_t)n * ldp;
   for (__nv_bfloat16** p : {&xh, &xl, &rh, &rl}) {
     if ((err = dev_malloc(p, plane * sizeof(__nv_bfloat16))) != cudaSuccess) return fail(err);
@@ -259,7 +425,7 @@ cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col,
   own.push_back(D);
   if ((err = dev_malloc(&rowsum, n * sizeof(double))) != cudaSuccess) return fail(err);
   own.push_back(rowsum);
-  if ((err = dev_malloc(&maxbits, sizeof(unsigned long long))) != cudaSuccess) return fail(err);
+  if ((err = dev_malloc(&maxbits, 2 * sizeof(unsigned long long))) != cudaSuccess) return fail(err);
   own.push_back(maxbits);
   if ((err = dev_malloc(&gerr, sizeof(int))) != cudaSuccess) return fail(err);
   own.push_back(gerr);
@@ -311,10 +477,17 @@ cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col,
   // the residual below is formed along rows as I - X M, which is R^T only for symmetric X
   symmetrize_inplace_kernel<<<sgrid, sblock, 0, s>>>(X, ldx, n);
   for (;; ++k) {
-    if (project) row_sum_kernel<<<n, 256, 0, s>>>(X, ldx, n, rowsum);
-    if ((err = cudaMemsetAsync(maxbits, 0, sizeof(unsigned long long), s)) != cudaSuccess) return fail(err);
-    {
+    if (project && !fixed) row_sum_kernel<<<n, 256, 0, s>>>(X, ldx, n, rowsum);
+    if ((err = cudaMemsetAsync(maxbits, 0, 2 * sizeof(unsigned long long), s)) != cudaSuccess) return fail(err);
+    if (fixed) {
       ProfScope prof("factor_ns_residual", 16.0 * (double)n * n, 0.0, s);
+      diag_max_kernel<<<std::min((n + 255) / 256, 64), 256, 0, s>>>(X, ldx, n, maxbits + 1);
+      // two or more rows share an SM up to 14000 cells; a longer row gets twice the threads
+      ns_residual_lap_kernel<<<n, n <= 14000 ? 512 : 1024, lap_smem, s>>>(
+          X, ldx, n, lap, maxbits + 1, alpha, reinterpret_cast<uint32_t*>(rh), reinterpret_cast<uint32_t*>(rl),
+          reinterpret_cast<uint32_t*>(xh), reinterpret_cast<uint32_t*>(xl), ldp, maxbits);
+    } else {
+      ProfScope prof("factor_ns_residual", 12.0 * (double)n * n, 0.0, s);
       dim3 grid(std::min((n + NSR_THREADS - 1) / NSR_THREADS, NSR_SPLIT), n);
       ns_residual_kernel<<<grid, NSR_THREADS, 0, s>>>(X, ldx, n, ptr, col, val, project ? rowsum : nullptr, alpha, rh, rl,
                                               ldp, maxbits);
@@ -331,7 +504,7 @@ cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col,
     }
     prev_plain = plain;
     if (k >= max_steps) break;
-    if ((err = split_bf16_f64(X, ldx, n, n, xh, xl, ldp, s)) != cudaSuccess) return fail(err);
+    if (!fixed && (err = split_bf16_f64(X, ldx, n, n, xh, xl, ldp, s)) != cudaSuccess) return fail(err);
     // D = X R' with B = R'^T stored row-major, R' = I - alpha M X; X R' is symmetric, so only the
     // tiles on and above the diagonal are computed; then X <- alpha (X + D)
     if ((err = gemm_bf16x3(&A, &B, nullptr, 1, n, n, n, D, ldp, false, gerr, s, 0, true)) != cudaSuccess)

@@ -456,9 +456,11 @@ cudaError_t dense_inverse_block_cg(const int32_t* ptr, const int32_t* col, const
                                    const AmgHierarchy* H, double tol, int max_iter, float* Xhi, float* Xlo,
                                    int* iters, cudaStream_t s, double* Xd = nullptr);
 // Newton-Schulz refinement of X ~ M^{-1} (k_factor.cu) for M = L + 1 1^T / n (project: writes
-// (Sigma^T Sigma)^+ = sym(X) - 1 1^T / n) or M = L (writes sym(X)) to the FP32 hi + lo planes.
-cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col, const double* val, int n,
-                                         bool project, double* X, long long ldx, int max_steps, double tol, float* Xhi,
+// (Sigma^T Sigma)^+ = sym(X) - 1 1^T / n) or M = L (writes sym(X)) to the FP32 hi + lo planes.  lap: L
+// as a graph Laplacian, or null: per row three neighbours, n where there is none, and the diagonal entry
+// (16 bits each, two rows a word; an odd n's last row is empty).
+cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col, const double* val, const uint4* lap,
+                                         int n, bool project, double* X, long long ldx, int max_steps, double tol, float* Xhi,
                                          float* Xlo, int* steps_done, double* final_residual, cudaStream_t s);
 // X = c D^{-1} for the diagonal D of a CSR matrix (n x n, row stride ldx; the rest of X zeroed)
 cudaError_t jacobi_start(const int32_t* ptr, const int32_t* col, const double* val, int n, double c, double* X,
