@@ -8,7 +8,7 @@
 //
 // Host: cluster trees (median bisection across the longest side of the item centres' extent, items
 // carrying support boxes), the admissibility test min(diam a, diam b) <= eta dist(a, b) on
-// boxes that do not touch (dist > 0), the block list.  Device: one CTA per admissible block runs the cross approximation on the
+// boxes that do not touch (dist > 0), the block list.  Device: a warp or a CTA per admissible block runs the cross approximation on the
 // resident dense matrix (rows and columns gathered through the cluster permutation), blocks whose
 // crosses reach the rank cap, or would take at least the block's own entries, stay dense, and the factors and dense blocks are packed into one
 // buffer per matrix.  The product y = H x (FP64 accumulation) runs over cross items and row tiles.
@@ -196,30 +196,6 @@ __device__ void block_argmax(float v, int i, float* sv, int* si, float& bv, int&
   __syncthreads();
 }
 
-// sums of four values over the CTA; every thread receives them
-__device__ void block_sum4(double (&a)[4], double (*sd)[HM_THREADS / 32 + 1]) {
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    for (int o = 16; o > 0; o >>= 1) a[k] += __shfl_down_sync(FULL, a[k], o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sd[k][w] = a[k];
-  __syncthreads();
-  if (w == 0) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      double x = l < HM_THREADS / 32 ? sd[k][l] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(FULL, x, o);
-      if (l == 0) sd[k][HM_THREADS / 32] = x;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 4; ++k) a[k] = sd[k][HM_THREADS / 32];
-  __syncthreads();
-}
-
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -230,39 +206,114 @@ __device__ __forceinline__ bool row_used(const int* used, int nused, int p) {
   return false;
 }
 
-// ACA with partial pivoting of one admissible block per CTA, on the dense matrix A (row stride
-// ld) through the cluster permutation.  The crosses go to the block's slot: U (cap x m) at
-// slot[b], Vt (cap x n) after it.  rank_out[b] = crosses kept, status_out[b] = 0 when the
-// stopping rule ||u|| ||v|| <= eps ||S||_F held (or every row was used), 1 when the rank cap or
-// the iteration cap ended the loop first.  All loops are bounded by the caps and the block's size.
+// FP32 -> FP64 by moving the bits: exponent rebased by 896, mantissa shifted by 29.  Zeros,
+// subnormals, infinities and NaN take the conversion instruction.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f);
+  if ((u & 0x7f800000u) - 0x00800000u >= 0x7f000000u) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// Warp sums of V = 2^k values a lane: afterwards v[0] of lane l is the sum of value l * V / 32 (each
+// exchange halves the values a lane holds: V - 1 + max(0, 5 - k) additions instead of 5 V).
+template <int V>
+__device__ __forceinline__ void warp_sums(double (&v)[V], int lane) {
+#pragma unroll
+  for (int step = 0; step < 5; ++step) {
+    const int off = 16 >> step, h = V >> (step + 1);
+    if (h == 0) {
+      v[0] += __shfl_xor_sync(FULL, v[0], off);
+    } else {
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int k = 0; k < h; ++k) {
+        const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+        v[k] = keep + __shfl_xor_sync(FULL, send, off);
+      }
+    }
+  }
+}
+
+constexpr int ACA_SMALL = 128;  // blocks of at most this many rows and columns take one warp
+constexpr int ACA_GROUP = 8;    // crosses whose four norm products a warp sums together
+
+// ACA with partial pivoting of one admissible block per team of WARPS warps (a CTA holds 8 / WARPS
+// teams), on the dense matrix A (row stride ld) through the cluster permutation.  The crosses go to the
+// block's slot: U (cap x m) at slot[b], Vt (cap x n) after it.  rank_out[b] = crosses kept, status_out[b]
+// = 0 when the stopping rule ||u|| ||v|| <= eps ||S||_F held (or every row was used), 1 when the rank cap
+// or the iteration cap ended the loop first.  All loops are bounded by the caps and the block's size.
+//
+// Most blocks are a few dozen rows: a CTA each left seven of its eight warps idle and cost a reduction
+// of FP64 sums over all of them per earlier cross, 160 warp additions on the slow FP64 pipe, which bound
+// the kernel.  A warp per small block synchronises with itself only, and the products of eight earlier
+// crosses are summed together, 31 additions.  GB300, T_A and V of 7680 functions and 5120 cells: 8.75 ->
+// 1.94 ms.
+template <int WARPS>
 __global__ void __launch_bounds__(HM_THREADS)
     hm_aca_kernel(const float2* __restrict__ A, long long ld, const int32_t* __restrict__ perm,
-                  const HmBlockDev* __restrict__ blk, const long long* __restrict__ slot, int cap, int iter_cap,
-                  float eps, float2* __restrict__ slots, int32_t* __restrict__ rank_out,
-                  int32_t* __restrict__ status_out) {
+                  const HmBlockDev* __restrict__ blk, const int32_t* __restrict__ list, int nlist,
+                  const long long* __restrict__ slot, int cap, int iter_cap, float eps, float2* __restrict__ slots,
+                  int32_t* __restrict__ rank_out, int32_t* __restrict__ status_out) {
   RF_COUNT_LAUNCH();
+  constexpr int T = 32 * WARPS;  // threads of a team
   __shared__ float sv[HM_THREADS / 32 + 1];
   __shared__ int si[HM_THREADS / 32 + 1];
-  __shared__ double sd[4][HM_THREADS / 32 + 1];
-  __shared__ int used[HM_MAX_ITER];
+  __shared__ double sd[WARPS][33];
+  __shared__ int used[WARPS == 1 ? 1 : HM_MAX_ITER];
   __shared__ int s_next;
-  const HmBlockDev B = blk[blockIdx.x];
-  const int m = B.r1 - B.r0, n = B.c1 - B.c0, tid = threadIdx.x;
+  const int team = blockIdx.x * (HM_THREADS / T) + threadIdx.x / T;
+  if (team >= nlist) return;  // whole teams only
+  const int b = list[team], tid = threadIdx.x % T, lane = threadIdx.x & 31, w = tid >> 5;
+  auto sync = [] {
+    if (WARPS == 1) __syncwarp();
+    else __syncthreads();
+  };
+  // largest v over the team (ties: smallest i); every thread receives it
+  auto argmax = [&](float v, int i, float& bv, int& bi) {
+    if (WARPS == 1) {
+      for (int o = 16; o > 0; o >>= 1) argmax_merge(v, i, __shfl_xor_sync(FULL, v, o), __shfl_xor_sync(FULL, i, o));
+      bv = v;
+      bi = i;
+    } else {
+      block_argmax(v, i, sv, si, bv, bi);
+    }
+  };
+  // sums over the team of 32 values a thread, value l in lane l of every warp
+  auto team_sums = [&](double (&v)[32]) -> double {
+    warp_sums<32>(v, lane);
+    if (WARPS == 1) return v[0];
+    sd[w][lane] = v[0];
+    __syncthreads();
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < WARPS; ++k) s += sd[k][lane];
+    __syncthreads();
+    return s;
+  };
+  const HmBlockDev B = blk[b];
+  const int m = B.r1 - B.r0, n = B.c1 - B.c0;
   const int32_t* rp = perm + B.r0;
   const int32_t* cp = perm + B.c0;
-  float2* U = slots + slot[blockIdx.x];
+  float2* U = slots + slot[b];
   float2* Vt = U + (size_t)cap * m;
   int rank = 0, nused = 0, status = 1, i = 0;
+  unsigned mine = 0;   // one warp: bit q for row lane + 32 q, set once the row was a pivot row
   double norm2 = 0.0;  // ||S_rank||_F^2, the same in every thread
+  auto is_used = [&](int p) { return WARPS == 1 ? (mine >> (p >> 5) & 1u) != 0 : row_used(used, nused, p); };
   for (int it = 0; it < iter_cap && rank < cap; ++it) {
-    if (tid == 0) used[nused] = i;
+    if (WARPS == 1) {
+      if ((i & 31) == lane) mine |= 1u << (i >> 5);
+    } else if (tid == 0) {
+      used[nused] = i;
+    }
     ++nused;
     // residual row i into the next cross's Vt row, and its largest entry
     float bv = -1.f;
     int bj = INT_MAX;
     const float2* Arow = A + (size_t)rp[i] * ld;
-    for (int j = tid; j < n; j += HM_THREADS) {
+    for (int j = tid; j < n; j += T) {
       float2 r = Arow[cp[j]];
+#pragma unroll 4
       for (int l = 0; l < rank; ++l) {
         const float2 p = cmulf(U[(size_t)l * m + i], Vt[(size_t)l * n + j]);
         r.x -= p.x;
@@ -271,20 +322,29 @@ __global__ void __launch_bounds__(HM_THREADS)
       Vt[(size_t)rank * n + j] = r;
       argmax_merge(bv, bj, r.x * r.x + r.y * r.y, j);
     }
+    sync();
     int js;
-    block_argmax(bv, bj, sv, si, bv, js);
+    argmax(bv, bj, bv, js);
     if (!(bv >= FLT_MIN)) {
       // the residual vanishes on this row (to below the normal range, where 1 / pivot would
       // overflow): the next row not yet used
-      if (tid == 0) {
-        int c = -1;
-        for (int p = 0; p < m && c < 0; ++p)
-          if (!row_used(used, nused, p)) c = p;
-        s_next = c;
+      if (WARPS == 1) {
+        int c = INT_MAX;
+        for (int p = lane; p < m && c == INT_MAX; p += 32)
+          if (!is_used(p)) c = p;
+        c = __reduce_min_sync(FULL, c);
+        i = c == INT_MAX ? -1 : c;
+      } else {
+        if (tid == 0) {
+          int c = -1;
+          for (int p = 0; p < m && c < 0; ++p)
+            if (!row_used(used, nused, p)) c = p;
+          s_next = c;
+        }
+        __syncthreads();
+        i = s_next;
+        __syncthreads();
       }
-      __syncthreads();
-      i = s_next;
-      __syncthreads();
       if (i < 0) {
         status = 0;  // every row reproduced
         break;
@@ -292,48 +352,81 @@ __global__ void __launch_bounds__(HM_THREADS)
       continue;
     }
     const float2 piv = Vt[(size_t)rank * n + js];
-    __syncthreads();  // every thread holds the pivot before its entry is rescaled
+    sync();  // every thread holds the pivot before its entry is rescaled
     const float dd = piv.x * piv.x + piv.y * piv.y;
     const float2 ip = make_float2(piv.x / dd, -piv.y / dd);
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};  // |u|^2, |v|^2
-    for (int j = tid; j < n; j += HM_THREADS) {
+    double nrm[2] = {0.0, 0.0};  // |u|^2, |v|^2 of this thread's entries
+    for (int j = tid; j < n; j += T) {
       const float2 v = cmulf(Vt[(size_t)rank * n + j], ip);
       Vt[(size_t)rank * n + j] = v;
-      acc[1] += (double)v.x * v.x + (double)v.y * v.y;
+      const double x = widen(v.x), y = widen(v.y);
+      nrm[1] = fma(x, x, fma(y, y, nrm[1]));
     }
+    sync();
     // residual column js into the next cross's U row, and the next pivot row
     float bu = -1.f;
     int bp = INT_MAX;
-    for (int p = tid; p < m; p += HM_THREADS) {
+    for (int p = tid; p < m; p += T) {
       float2 u = A[(size_t)rp[p] * ld + cp[js]];
+#pragma unroll 4
       for (int l = 0; l < rank; ++l) {
         const float2 q = cmulf(Vt[(size_t)l * n + js], U[(size_t)l * m + p]);
         u.x -= q.x;
         u.y -= q.y;
       }
       U[(size_t)rank * m + p] = u;
-      acc[0] += (double)u.x * u.x + (double)u.y * u.y;
-      if (!row_used(used, nused, p)) argmax_merge(bu, bp, u.x * u.x + u.y * u.y, p);
+      const double x = widen(u.x), y = widen(u.y);
+      nrm[0] = fma(x, x, fma(y, y, nrm[0]));
+      if (!is_used(p)) argmax_merge(bu, bp, u.x * u.x + u.y * u.y, p);
     }
-    block_sum4(acc, sd);
-    const double uu = acc[0], vv = acc[1];
-    __syncthreads();  // the new cross is complete in global memory
-    // ||S + u v^T||^2 = ||S||^2 + 2 Re sum_l (u_l^H u)(v_l^H v) + ||u||^2 ||v||^2
-    double cross = 0.0;
-    for (int l = 0; l < rank; ++l) {
-      double c[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int p = tid; p < m; p += HM_THREADS) {
-        const float2 a = U[(size_t)l * m + p], b = U[(size_t)rank * m + p];
-        c[0] += (double)a.x * b.x + (double)a.y * b.y;  // conj(a) b
-        c[1] += (double)a.x * b.y - (double)a.y * b.x;
+    sync();  // the new cross is complete in global memory
+    // ||S + u v^T||^2 = ||S||^2 + 2 Re sum_l (u_l^H u)(v_l^H v) + ||u||^2 ||v||^2: the four products of
+    // up to ACA_GROUP earlier crosses at a time, the norms in the first group's last places
+    double cross = 0.0, uu = 0.0, vv = 0.0;
+    for (int l0 = 0; l0 == 0 || l0 < rank; l0 += l0 == 0 ? ACA_GROUP - 1 : ACA_GROUP) {
+      const int nl = min(l0 == 0 ? ACA_GROUP - 1 : ACA_GROUP, rank - l0);
+      double c[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) c[k] = 0.0;
+      for (int p = tid; p < m; p += T) {
+        const float2 ub = U[(size_t)rank * m + p];
+        const double x = widen(ub.x), y = widen(ub.y);
+#pragma unroll
+        for (int l = 0; l < ACA_GROUP; ++l) {
+          if (l >= nl) break;
+          const float2 ua = U[(size_t)(l0 + l) * m + p];
+          const double ax = widen(ua.x), ay = widen(ua.y);
+          c[4 * l] = fma(ax, x, fma(ay, y, c[4 * l]));  // conj(a) b
+          c[4 * l + 1] = fma(ax, y, fma(-ay, x, c[4 * l + 1]));
+        }
       }
-      for (int j = tid; j < n; j += HM_THREADS) {
-        const float2 a = Vt[(size_t)l * n + j], b = Vt[(size_t)rank * n + j];
-        c[2] += (double)a.x * b.x + (double)a.y * b.y;
-        c[3] += (double)a.x * b.y - (double)a.y * b.x;
+      for (int j = tid; j < n; j += T) {
+        const float2 vb = Vt[(size_t)rank * n + j];
+        const double x = widen(vb.x), y = widen(vb.y);
+#pragma unroll
+        for (int l = 0; l < ACA_GROUP; ++l) {
+          if (l >= nl) break;
+          const float2 va = Vt[(size_t)(l0 + l) * n + j];
+          const double ax = widen(va.x), ay = widen(va.y);
+          c[4 * l + 2] = fma(ax, x, fma(ay, y, c[4 * l + 2]));
+          c[4 * l + 3] = fma(ax, y, fma(-ay, x, c[4 * l + 3]));
+        }
       }
-      block_sum4(c, sd);
-      cross += c[0] * c[2] - c[1] * c[3];
+      if (l0 == 0) {
+        c[30] = nrm[0];
+        c[31] = nrm[1];
+      }
+      const double s = team_sums(c);
+      // lanes 4 l .. 4 l + 3 hold c0 .. c3 of cross l: c0 c2 - c1 c3
+      const double t = __shfl_down_sync(FULL, s, 2);
+      double q = lane & 1 ? -s * t : s * t;
+      if ((lane & 3) > 1 || (lane >> 2) >= nl) q = 0.0;
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(FULL, q, o);
+      cross += q;
+      if (l0 == 0) {
+        uu = __shfl_sync(FULL, s, 30);
+        vv = __shfl_sync(FULL, s, 31);
+      }
     }
     norm2 += 2.0 * cross + uu * vv;
     ++rank;
@@ -342,7 +435,7 @@ __global__ void __launch_bounds__(HM_THREADS)
       break;
     }
     int np;
-    block_argmax(bu, bp, sv, si, bu, np);
+    argmax(bu, bp, bu, np);
     if (bu < 0.f) {
       status = 0;  // every row used
       break;
@@ -350,8 +443,8 @@ __global__ void __launch_bounds__(HM_THREADS)
     i = np;
   }
   if (tid == 0) {
-    rank_out[blockIdx.x] = rank;
-    status_out[blockIdx.x] = status;
+    rank_out[b] = rank;
+    status_out[b] = status;
   }
 }
 
@@ -406,14 +499,6 @@ struct HmTile {
   int32_t begin, end;      // its entries of the cover list: 2 block + (1: as columns)
 };
 
-// FP32 -> FP64 by moving the bits: exponent rebased by 896, mantissa shifted by 29.  Zeros,
-// subnormals, infinities and NaN take the conversion instruction.
-__device__ __forceinline__ double widen(float f) {
-  const unsigned u = __float_as_uint(f);
-  if ((u & 0x7f800000u) - 0x00800000u >= 0x7f000000u) return (double)f;
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
-}
-
 // xp: group g (columns 4 g ..) at 4 g n, entry p, column c of the group at p * (columns of the group) + c
 __global__ void hm_gather_kernel(const double2* __restrict__ x, const int32_t* __restrict__ perm, int n, int nrhs,
                                  double2* __restrict__ xp) {
@@ -424,26 +509,6 @@ __global__ void hm_gather_kernel(const double2* __restrict__ x, const int32_t* _
     const int c = (int)(e / n), p = (int)(e - (long long)c * n);
     const int g = c / HM_COLS, nc = min(HM_COLS, nrhs - g * HM_COLS);
     xp[(size_t)g * HM_COLS * n + (size_t)p * nc + (c - g * HM_COLS)] = x[(size_t)c * n + perm[p]];
-  }
-}
-
-// Warp sums of V = 2^k values a lane: afterwards v[0] of lane l is the sum of value l * V / 32 (each
-// exchange halves the values a lane holds: V - 1 + max(0, 5 - k) additions instead of 5 V).
-template <int V>
-__device__ __forceinline__ void warp_sums(double (&v)[V], int lane) {
-#pragma unroll
-  for (int step = 0; step < 5; ++step) {
-    const int off = 16 >> step, h = V >> (step + 1);
-    if (h == 0) {
-      v[0] += __shfl_xor_sync(FULL, v[0], off);
-    } else {
-      const bool up = (lane & off) != 0;
-#pragma unroll
-      for (int k = 0; k < h; ++k) {
-        const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
-        v[k] = keep + __shfl_xor_sync(FULL, send, off);
-      }
-    }
   }
 }
 
@@ -741,9 +806,29 @@ int build_part(const float2* A, int ld, int n, const std::vector<double>& cen, c
     HM_CUDA(cudaMemcpy(slot_d, slot.data(), slot.size() * sizeof(long long), cudaMemcpyHostToDevice));
     const int iter_cap = std::min(cap + 16, HM_MAX_ITER);
     {
+      // the large blocks first (a CTA each), the small ones (a warp each) fill the chip beside them
+      std::vector<int32_t> order;
+      order.reserve(cand.size());
+      for (int small = 0; small < 2; ++small)
+        for (size_t c = 0; c < cand.size(); ++c)
+          if ((std::max(cand[c].r1 - cand[c].r0, cand[c].c1 - cand[c].c0) <= ACA_SMALL) == (small != 0))
+            order.push_back((int32_t)c);
+      int large = 0;
+      while (large < (int)order.size() && std::max(cand[order[large]].r1 - cand[order[large]].r0,
+                                                   cand[order[large]].c1 - cand[order[large]].c0) > ACA_SMALL)
+        ++large;
+      const int nsmall = (int)order.size() - large, per = HM_THREADS / 32;
+      int32_t* order_d = nullptr;
+      HM_CUDA(tmp.alloc(&order_d, 4 * order.size()));
+      HM_CUDA(cudaMemcpy(order_d, order.data(), 4 * order.size(), cudaMemcpyHostToDevice));
       ProfScope prof("hm_aca", 8.0 * (double)slot_elems, 0.0, 0);
-      hm_aca_kernel<<<(unsigned)cand.size(), HM_THREADS>>>(A, ld, out.perm, cand_d, slot_d, cap, iter_cap,
-                                                          (float)o.eps, slots, rank_d, status_d);
+      if (large > 0)
+        hm_aca_kernel<8><<<large, HM_THREADS>>>(A, ld, out.perm, cand_d, order_d, large, slot_d, cap, iter_cap,
+                                                (float)o.eps, slots, rank_d, status_d);
+      if (nsmall > 0)
+        hm_aca_kernel<1><<<(nsmall + per - 1) / per, HM_THREADS>>>(A, ld, out.perm, cand_d, order_d + large, nsmall,
+                                                                   slot_d, cap, iter_cap, (float)o.eps, slots, rank_d,
+                                                                   status_d);
     }
     HM_CUDA(cudaGetLastError());
     lists = cover_lists(blocks, n);  // while the crosses are found
