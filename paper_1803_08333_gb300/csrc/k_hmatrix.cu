@@ -20,9 +20,13 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <future>
 #include <memory>
 #include <mutex>
+#include <new>
 #include <string>
+#include <system_error>
+#include <utility>
 #include <vector>
 
 #include "rfcmp_internal.h"
@@ -38,17 +42,13 @@ struct HmNode {
   int start = 0, stop = 0;
   double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
   int child[2] = {-1, -1};
-  double diam() const {
-    double s = 0.0;
-    for (int d = 0; d < 3; ++d) s += (hi[d] - lo[d]) * (hi[d] - lo[d]);
-    return std::sqrt(s);
-  }
+  double diam = 0.0;  // of the box
 };
 
 // Recursive bisection: a cluster of more than `leaf` items is sorted (stably) along the axis of
 // the largest extent of its item centres and split at the middle position.
 int build_tree(const double* cen, const double* slo, const double* shi, int start, int stop, int leaf,
-               std::vector<int32_t>& perm, std::vector<HmNode>& nodes) {
+               std::vector<int32_t>& perm, std::vector<HmNode>& nodes, std::vector<std::pair<double, int32_t>>& keys) {
   const int id = (int)nodes.size();
   nodes.emplace_back();
   HmNode node;
@@ -68,15 +68,22 @@ int build_tree(const double* cen, const double* slo, const double* shi, int star
       chi[d] = std::max(chi[d], cen[3 * i + d]);
     }
   }
+  {
+    double d2 = 0.0;
+    for (int d = 0; d < 3; ++d) d2 += (node.hi[d] - node.lo[d]) * (node.hi[d] - node.lo[d]);
+    node.diam = std::sqrt(d2);
+  }
   if (stop - start > leaf) {
     int axis = 0;  // the first axis of the largest extent
     for (int d = 1; d < 3; ++d)
       if (chi[d] - clo[d] > chi[axis] - clo[axis]) axis = d;
-    std::stable_sort(perm.begin() + start, perm.begin() + stop,
-                     [&](int32_t a, int32_t b) { return cen[3 * a + axis] < cen[3 * b + axis]; });
+    keys.resize(stop - start);  // (coordinate, item): the sort reads each coordinate once
+    for (int p = start; p < stop; ++p) keys[p - start] = {cen[3 * perm[p] + axis], perm[p]};
+    std::stable_sort(keys.begin(), keys.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
+    for (int p = start; p < stop; ++p) perm[p] = keys[p - start].second;
     const int mid = start + (stop - start) / 2;
-    node.child[0] = build_tree(cen, slo, shi, start, mid, leaf, perm, nodes);
-    node.child[1] = build_tree(cen, slo, shi, mid, stop, leaf, perm, nodes);
+    node.child[0] = build_tree(cen, slo, shi, start, mid, leaf, perm, nodes, keys);
+    node.child[1] = build_tree(cen, slo, shi, mid, stop, leaf, perm, nodes, keys);
   }
   nodes[id] = node;
   return id;
@@ -109,7 +116,7 @@ std::vector<HmBlockHost> block_list(const std::vector<HmNode>& nodes, double eta
     const HmNode &a = nodes[ia], &b = nodes[ib];
     if (a.start > b.start) continue;  // below the diagonal: the transpose of a mirrored block
     const double dist = box_distance(a, b);
-    if (dist > 0.0 && std::min(a.diam(), b.diam()) <= eta * dist) {  // boxes that touch: never
+    if (dist > 0.0 && std::min(a.diam, b.diam) <= eta * dist) {  // boxes that touch: never
       out.push_back({a.start, a.stop, b.start, b.stop, 1});
     } else if (a.child[0] < 0 && b.child[0] < 0) {
       out.push_back({a.start, a.stop, b.start, b.stop, 0});
@@ -139,7 +146,8 @@ void partition(const double* cen, const double* slo, const double* shi, int n, i
   perm.resize(n);
   for (int i = 0; i < n; ++i) perm[i] = i;
   std::vector<HmNode> nodes;
-  if (n > 0) build_tree(cen, slo, shi, 0, n, leaf, perm, nodes);
+  std::vector<std::pair<double, int32_t>> keys;
+  if (n > 0) build_tree(cen, slo, shi, 0, n, leaf, perm, nodes, keys);
   blocks = block_list(nodes, eta);
 }
 
@@ -753,98 +761,98 @@ cudaError_t keep(T** d, const std::vector<T>& h, std::vector<void*>& owned) {
   return h.empty() ? cudaSuccess : cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
 }
 
-// Compresses the dense n x n matrix A (row stride ld, both triangles stored) whose items have the
-// given centres and support boxes.  owned receives the part's device buffers; budget_left bounds
-// the bytes it may hold at the peak of the build.
-int build_part(const float2* A, int ld, int n, const std::vector<double>& cen, const std::vector<double>& lo,
-               const std::vector<double>& hi, const rfcmp_hm_opts& o, uint64_t budget_left, HmPart& out,
-               std::vector<void*>& owned) {
-  out.n = n;
+// One matrix on its way to the compressed form: the partition (host), the cross approximations (queued
+// on the legacy stream) and what the packing reads.
+struct PartBuild {
   std::vector<int32_t> perm;
   std::vector<HmBlockHost> blocks;
-  partition(cen.data(), lo.data(), hi.data(), n, o.leaf, o.eta, perm, blocks);
-  const int cap = o.max_rank;
-  std::vector<HmBlockDev> cand;
+  std::vector<HmBlockDev> cand;  // the admissible blocks
   std::vector<long long> slot;
-  long long slot_elems = 0, dense_elems = 0;
-  for (const HmBlockHost& b : blocks) {
-    const long long m = b.r1 - b.r0, nn = b.c1 - b.c0;
-    if (b.admissible) {
-      cand.push_back({b.r0, b.r1, b.c0, b.c1, 0, 0, 0});
-      slot.push_back(slot_elems);
+  int32_t *rank_d = nullptr, *status_d = nullptr;
+  float2* slots = nullptr;
+  HmTemps tmp;
+};
+
+// Queues the cross approximations of the dense n x n matrix A (row stride ld, both triangles stored)
+// partitioned in b.  owned receives the part's device buffers; budget_left bounds the bytes it may hold
+// at the peak of the build.
+int start_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, uint64_t budget_left, PartBuild& b, HmPart& out,
+               std::vector<void*>& owned) {
+  out.n = n;
+  const int cap = o.max_rank;
+  std::vector<int32_t> order;  // candidates, the large ones (a CTA each) before the small ones (a warp each)
+  long long slot_elems = 0, worst = 0;
+  for (const HmBlockHost& h : b.blocks) {
+    const long long m = h.r1 - h.r0, nn = h.c1 - h.c0;
+    worst += m * nn;  // the peak holds the slots and, at worst, every block dense
+    if (h.admissible) {
+      b.cand.push_back({h.r0, h.r1, h.c0, h.c1, 0, 0, 0});
+      b.slot.push_back(slot_elems);
       slot_elems += (long long)cap * (m + nn);
-    } else {
-      dense_elems += m * nn;
     }
   }
-  // the peak holds the slots and, at worst, every block dense
-  long long worst = dense_elems;
-  for (const HmBlockDev& c : cand) worst += (long long)(c.r1 - c.r0) * (c.c1 - c.c0);
-  const uint64_t peak = 8ull * (uint64_t)(slot_elems + worst) + 64ull * blocks.size() + 4ull * n;
+  const uint64_t peak = 8ull * (uint64_t)(slot_elems + worst) + 64ull * b.blocks.size() + 4ull * n;
   if (budget_left != UINT64_MAX && peak > budget_left)
     return set_error(RFCMP_ERR_OUT_OF_BUDGET, "compression needs up to " + std::to_string(peak) + " bytes, budget has " +
                                                   std::to_string(budget_left));
-  HmTemps tmp;
   HM_CUDA(dev_malloc(&out.perm, std::max<size_t>(4 * (size_t)n, 4)));
   owned.push_back(out.perm);
-  if (n > 0) HM_CUDA(cudaMemcpy(out.perm, perm.data(), 4 * (size_t)n, cudaMemcpyHostToDevice));
-  std::vector<int32_t> rank(cand.size(), 0), status(cand.size(), 1);
-  float2* slots = nullptr;
+  if (n > 0) HM_CUDA(cudaMemcpy(out.perm, b.perm.data(), 4 * (size_t)n, cudaMemcpyHostToDevice));
+  if (b.cand.empty()) return RFCMP_OK;
+  auto is_small = [&](const HmBlockDev& c) { return std::max(c.r1 - c.r0, c.c1 - c.c0) <= ACA_SMALL; };
+  order.reserve(b.cand.size());
+  for (size_t c = 0; c < b.cand.size(); ++c)
+    if (!is_small(b.cand[c])) order.push_back((int32_t)c);
+  const int large = (int)order.size(), small = (int)b.cand.size() - large, per = HM_THREADS / 32;
+  for (size_t c = 0; c < b.cand.size(); ++c)
+    if (is_small(b.cand[c])) order.push_back((int32_t)c);
+  HmBlockDev* cand_d = nullptr;
   long long* slot_d = nullptr;
-  CoverLists lists;
-  if (cand.empty()) {
-    lists = cover_lists(blocks, n);
-  } else {
-    HmBlockDev* cand_d = nullptr;
-    int32_t *rank_d = nullptr, *status_d = nullptr;
-    HM_CUDA(tmp.alloc(&cand_d, cand.size() * sizeof(HmBlockDev)));
-    HM_CUDA(tmp.alloc(&slot_d, slot.size() * sizeof(long long)));
-    HM_CUDA(tmp.alloc(&slots, 8 * (size_t)slot_elems));
-    HM_CUDA(tmp.alloc(&rank_d, 4 * cand.size()));
-    HM_CUDA(tmp.alloc(&status_d, 4 * cand.size()));
-    HM_CUDA(cudaMemcpy(cand_d, cand.data(), cand.size() * sizeof(HmBlockDev), cudaMemcpyHostToDevice));
-    HM_CUDA(cudaMemcpy(slot_d, slot.data(), slot.size() * sizeof(long long), cudaMemcpyHostToDevice));
-    const int iter_cap = std::min(cap + 16, HM_MAX_ITER);
-    {
-      // the large blocks first (a CTA each), the small ones (a warp each) fill the chip beside them
-      std::vector<int32_t> order;
-      order.reserve(cand.size());
-      for (int small = 0; small < 2; ++small)
-        for (size_t c = 0; c < cand.size(); ++c)
-          if ((std::max(cand[c].r1 - cand[c].r0, cand[c].c1 - cand[c].c0) <= ACA_SMALL) == (small != 0))
-            order.push_back((int32_t)c);
-      int large = 0;
-      while (large < (int)order.size() && std::max(cand[order[large]].r1 - cand[order[large]].r0,
-                                                   cand[order[large]].c1 - cand[order[large]].c0) > ACA_SMALL)
-        ++large;
-      const int nsmall = (int)order.size() - large, per = HM_THREADS / 32;
-      int32_t* order_d = nullptr;
-      HM_CUDA(tmp.alloc(&order_d, 4 * order.size()));
-      HM_CUDA(cudaMemcpy(order_d, order.data(), 4 * order.size(), cudaMemcpyHostToDevice));
-      ProfScope prof("hm_aca", 8.0 * (double)slot_elems, 0.0, 0);
-      if (large > 0)
-        hm_aca_kernel<8><<<large, HM_THREADS>>>(A, ld, out.perm, cand_d, order_d, large, slot_d, cap, iter_cap,
-                                                (float)o.eps, slots, rank_d, status_d);
-      if (nsmall > 0)
-        hm_aca_kernel<1><<<(nsmall + per - 1) / per, HM_THREADS>>>(A, ld, out.perm, cand_d, order_d + large, nsmall,
-                                                                   slot_d, cap, iter_cap, (float)o.eps, slots, rank_d,
-                                                                   status_d);
-    }
-    HM_CUDA(cudaGetLastError());
-    lists = cover_lists(blocks, n);  // while the crosses are found
-    HM_CUDA(cudaMemcpy(rank.data(), rank_d, 4 * cand.size(), cudaMemcpyDeviceToHost));
-    HM_CUDA(cudaMemcpy(status.data(), status_d, 4 * cand.size(), cudaMemcpyDeviceToHost));
+  int32_t* order_d = nullptr;
+  HM_CUDA(b.tmp.alloc(&cand_d, b.cand.size() * sizeof(HmBlockDev)));
+  HM_CUDA(b.tmp.alloc(&slot_d, b.slot.size() * sizeof(long long)));
+  HM_CUDA(b.tmp.alloc(&order_d, 4 * order.size()));
+  HM_CUDA(b.tmp.alloc(&b.slots, 8 * (size_t)slot_elems));
+  HM_CUDA(b.tmp.alloc(&b.rank_d, 4 * b.cand.size()));
+  HM_CUDA(b.tmp.alloc(&b.status_d, 4 * b.cand.size()));
+  HM_CUDA(cudaMemcpy(cand_d, b.cand.data(), b.cand.size() * sizeof(HmBlockDev), cudaMemcpyHostToDevice));
+  HM_CUDA(cudaMemcpy(slot_d, b.slot.data(), b.slot.size() * sizeof(long long), cudaMemcpyHostToDevice));
+  HM_CUDA(cudaMemcpy(order_d, order.data(), 4 * order.size(), cudaMemcpyHostToDevice));
+  const int iter_cap = std::min(cap + 16, HM_MAX_ITER);
+  ProfScope prof("hm_aca", 8.0 * (double)slot_elems, 0.0, 0);
+  if (large > 0)
+    hm_aca_kernel<8><<<large, HM_THREADS>>>(A, ld, out.perm, cand_d, order_d, large, slot_d, cap, iter_cap,
+                                            (float)o.eps, b.slots, b.rank_d, b.status_d);
+  if (small > 0)
+    hm_aca_kernel<1><<<(small + per - 1) / per, HM_THREADS>>>(A, ld, out.perm, cand_d, order_d + large, small, slot_d,
+                                                              cap, iter_cap, (float)o.eps, b.slots, b.rank_d,
+                                                              b.status_d);
+  HM_CUDA(cudaGetLastError());
+  return RFCMP_OK;
+}
+
+// Waits for the cross approximations and packs the final blocks: the admissible ones whose crosses met the
+// stopping rule in low rank, the rest dense.
+int finish_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, PartBuild& b, HmPart& out,
+                std::vector<void*>& owned) {
+  const int cap = o.max_rank;
+  const CoverLists lists = cover_lists(b.blocks, n);  // while the crosses are found
+  std::vector<int32_t> rank(b.cand.size(), 0), status(b.cand.size(), 1);
+  if (!b.cand.empty()) {
+    HM_CUDA(cudaMemcpy(rank.data(), b.rank_d, 4 * b.cand.size(), cudaMemcpyDeviceToHost));
+    HM_CUDA(cudaMemcpy(status.data(), b.status_d, 4 * b.cand.size(), cudaMemcpyDeviceToHost));
   }
-  // final blocks: the admissible ones whose crosses met the stopping rule in low rank, the rest dense
   std::vector<HmBlockDev> fin;
   std::vector<long long> fin_slot;
+  fin.reserve(b.blocks.size());
+  fin_slot.reserve(b.blocks.size());
   long long off = 0;
   size_t ci = 0;
-  for (const HmBlockHost& b : blocks) {
-    const long long m = b.r1 - b.r0, nn = b.c1 - b.c0;
-    HmBlockDev d{b.r0, b.r1, b.c0, b.c1, -1, 0, off};
+  for (const HmBlockHost& h : b.blocks) {
+    const long long m = h.r1 - h.r0, nn = h.c1 - h.c0;
+    HmBlockDev d{h.r0, h.r1, h.c0, h.c1, -1, 0, off};
     long long s = 0;
-    if (b.admissible) {
+    if (h.admissible) {
       const size_t c = ci++;
       if (status[c] != 0 || rank[c] < 0 || rank[c] > cap) {
         ++out.n_capped;
@@ -854,7 +862,7 @@ int build_part(const float2* A, int ld, int n, const std::vector<double>& cen, c
         d.rank = rank[c];
         d.t0 = out.ncross;
         out.ncross += 2 * d.rank;
-        s = slot[c];
+        s = b.slot[c];
         ++out.n_lowrank;
         out.max_rank = std::max(out.max_rank, rank[c]);
       }
@@ -872,10 +880,10 @@ int build_part(const float2* A, int ld, int n, const std::vector<double>& cen, c
   owned.push_back(out.blocks);
   if (!fin.empty()) {
     long long* fslot_d = nullptr;
-    HM_CUDA(tmp.alloc(&fslot_d, fin_slot.size() * sizeof(long long)));
+    HM_CUDA(b.tmp.alloc(&fslot_d, fin_slot.size() * sizeof(long long)));
     HM_CUDA(cudaMemcpy(out.blocks, fin.data(), fin.size() * sizeof(HmBlockDev), cudaMemcpyHostToDevice));
     HM_CUDA(cudaMemcpy(fslot_d, fin_slot.data(), fin_slot.size() * sizeof(long long), cudaMemcpyHostToDevice));
-    hm_pack_kernel<<<(unsigned)fin.size(), HM_THREADS>>>(A, ld, out.perm, out.blocks, fslot_d, cap, slots, out.data);
+    hm_pack_kernel<<<(unsigned)fin.size(), HM_THREADS>>>(A, ld, out.perm, out.blocks, fslot_d, cap, b.slots, out.data);
     HM_CUDA(cudaGetLastError());
   }
   const std::vector<int2> items = cross_items(fin);
@@ -1008,21 +1016,43 @@ int rfcmp_hm_create(rfcmp_op* op, const rfcmp_hm_opts* opts_in, rfcmp_hm** out) 
   auto hm = std::make_unique<rfcmp_hm>();
   hm->device = v.device;
   hm->opts = o;
-  std::vector<double> ccen, clo, chi, ecen, elo, ehi;
-  supports(*v.top, v.verts, ccen, clo, chi, ecen, elo, ehi);
-  const float2* mats[2] = {v.TA, v.V};
-  const int lds[2] = {v.ldN, v.ldC}, ns[2] = {v.n, v.nc};
-  for (int w = 0; w < 2; ++w) {
-    uint64_t left = UINT64_MAX;
-    if (v.budget) {
-      const uint64_t used = v.ctx_bytes->load() + hm->bytes;
-      left = v.budget > used ? v.budget - used : 0;
+  try {
+    std::vector<double> ccen, clo, chi, ecen, elo, ehi;
+    supports(*v.top, v.verts, ccen, clo, chi, ecen, elo, ehi);
+    const float2* mats[2] = {v.TA, v.V};
+    const int lds[2] = {v.ldN, v.ldC}, ns[2] = {v.n, v.nc};
+    PartBuild part[2];
+    // the host partitions V beside T_A (a thread of its own, or after it where none can be had) and, where
+    // no budget orders the two, while T_A's crosses are found
+    auto split_v = [&] { partition(ccen.data(), clo.data(), chi.data(), v.nc, o.leaf, o.eta, part[1].perm, part[1].blocks); };
+    std::future<void> other;
+    try {
+      other = std::async(std::launch::async, split_v);
+    } catch (const std::system_error&) {
     }
-    rc = build_part(mats[w], lds[w], ns[w], w == 0 ? ecen : ccen, w == 0 ? elo : clo, w == 0 ? ehi : chi, o, left,
-                    hm->part[w], hm->owned);
-    if (rc != RFCMP_OK) return rc;
-    hm->bytes += hm->part[w].bytes;
+    partition(ecen.data(), elo.data(), ehi.data(), v.n, o.leaf, o.eta, part[0].perm, part[0].blocks);
+    const bool together = v.budget == 0;
+    for (int w = 0; w < 2 && rc == RFCMP_OK; ++w) {
+      uint64_t left = UINT64_MAX;
+      if (v.budget) {
+        const uint64_t used = v.ctx_bytes->load() + hm->bytes;
+        left = v.budget > used ? v.budget - used : 0;
+      }
+      if (w == 1) {
+        if (other.valid()) other.get();
+        else split_v();
+      }
+      rc = start_part(mats[w], lds[w], ns[w], o, left, part[w], hm->part[w], hm->owned);
+      if (rc != RFCMP_OK || (together && w == 0)) continue;
+      for (int z = together ? 0 : w; z <= w && rc == RFCMP_OK; ++z) {
+        rc = finish_part(mats[z], lds[z], ns[z], o, part[z], hm->part[z], hm->owned);
+        hm->bytes += hm->part[z].bytes;
+      }
+    }
+  } catch (const std::bad_alloc&) {
+    return set_error(RFCMP_ERR_CUDA, "out of host memory");
   }
+  if (rc != RFCMP_OK) return rc;
   hm->ctx_bytes = v.ctx_bytes;
   hm->ctx_live = v.ctx_live;
   *hm->ctx_bytes += hm->bytes;
