@@ -290,6 +290,35 @@ __global__ void symmetrize_inplace_kernel(double* __restrict__ X, long long ldx,
   }
 }
 
+// hi + lo <- (M + M^T) / 2 of M = hi + lo in place, tiles paired as above: a factor whose columns were solved one
+// by one is symmetric only to the solver's tolerance, and the streaming products read its upper triangle
+__global__ void symmetrize_planes_kernel(float* __restrict__ hi, float* __restrict__ lo, long long ld, int n) {
+  RF_COUNT_LAUNCH();
+  __shared__ double a[TT][TT + 1], b[TT][TT + 1];
+  const int bx = blockIdx.x, by = blockIdx.y;
+  if (by > bx) return;
+  const int r0 = by * TT, c0 = bx * TT;
+  auto get = [&](int i, int j) {
+    const size_t at = (size_t)i * ld + j;
+    return i < n && j < n ? (double)hi[at] + (double)lo[at] : 0.0;
+  };
+  auto put = [&](int i, int j, double v) {
+    if (i >= n || j >= n) return;
+    const float h = (float)v;
+    hi[(size_t)i * ld + j] = h;
+    lo[(size_t)i * ld + j] = (float)(v - (double)h);
+  };
+  for (int r = threadIdx.y; r < TT; r += blockDim.y) {
+    a[r][threadIdx.x] = get(r0 + r, c0 + threadIdx.x);
+    b[r][threadIdx.x] = get(c0 + r, r0 + threadIdx.x);
+  }
+  __syncthreads();
+  for (int r = threadIdx.y; r < TT; r += blockDim.y) {
+    put(r0 + r, c0 + threadIdx.x, 0.5 * (a[r][threadIdx.x] + b[threadIdx.x][r]));
+    put(c0 + r, r0 + threadIdx.x, 0.5 * (b[r][threadIdx.x] + a[threadIdx.x][r]));
+  }
+}
+
 // X <- alpha (X + D) for a symmetric D of which only the 128 x 128 tiles on or above the diagonal
 // were computed: block (bx, by), by <= bx, adds tile (by, bx) of D to X there and its transpose
 // to tile (bx, by); a diagonal tile adds (D + D^T) / 2, so X stays exactly symmetric.  !SCALED:
@@ -541,6 +570,12 @@ cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col,
   *steps_done = k;
   *final_residual = res;
   return fail(cudaSuccess);
+}
+
+cudaError_t symmetrize_planes(float* hi, float* lo, int n, int ld, cudaStream_t s) {
+  const dim3 grid((n + TT - 1) / TT, (n + TT - 1) / TT), block(TT, 8);
+  symmetrize_planes_kernel<<<grid, block, 0, s>>>(hi, lo, ld, n);
+  return cudaGetLastError();
 }
 
 RF_LAUNCH_READER(launches_factor)

@@ -334,13 +334,14 @@ cudaError_t gemv_c64_dispatch(const float2* M, int ld, int n, bool conj, GemvMod
   const int chunk = gemv_chunk(w);
   const int upr = (ld + chunk - 1) / chunk;
   const long long units = (long long)rowblocks * upr;
-  const bool stream = mode == GEMV_F32 && NR <= 2 && w.chunk == 0 && w.ctas_per_sm == 0 && w.err && w.symmetric;
+  const bool can = w.chunk == 0 && w.ctas_per_sm == 0 && w.err, sym = can && w.symmetric;
+  const bool stream = sym && mode == GEMV_F32 && NR <= 2, stream_ff = mode == GEMV_FF && (NR == 1 ? can : sym);
   // algorithmic bytes: the matrix (its upper triangle where the symmetric kernel reads only that)
   // plus the vectors
-  const double mbytes = stream ? 4.0 * n * (n + 1.0) : 8.0 * n * n;
+  const double mbytes = stream || (stream_ff && NR > 1) ? 4.0 * n * (n + 1.0) : 8.0 * n * n;
   ProfScope prof(mode == GEMV_FF ? "gemv_c64_ff" : "gemv_c64_f32", mbytes + 32.0 * n * NR, 8.0 * n * n * NR, s);
   if (stream) return gemv_stream_c64<NR <= 1 ? 1 : 2>(M, ld, n, conj, w, s);
-  if (NR == 1 && mode == GEMV_FF && w.chunk == 0 && w.ctas_per_sm == 0 && w.err) return gemv_stream_c64_ff(M, ld, n, conj, w, s);
+  if (stream_ff) return gemv_stream_c64_ff(M, ld, n, NR, conj, w, s);
 #define RF_LAUNCH_C(FFV, CJ)                                                                      \
   {                                                                                               \
     auto k = gemv_c64_kernel<NR, FFV, CJ>;                                                        \
@@ -363,10 +364,12 @@ cudaError_t gemv_r32_dispatch(const float* Mhi, const float* Mlo, int ld, int n,
   const int chunk = gemv_chunk(w);
   const int upr = (ld + chunk - 1) / chunk;
   const long long units = (long long)rowblocks * upr;
-  const bool stream = mode == GEMV_F32 && NR <= 2 && w.chunk == 0 && w.ctas_per_sm == 0 && w.err && w.symmetric;
-  const double mbytes = mode == GEMV_FF ? 8.0 * n * n : (stream ? 2.0 * n * (n + 1.0) : 4.0 * n * n);
+  const bool sym = w.chunk == 0 && w.ctas_per_sm == 0 && w.err && w.symmetric;
+  const bool stream = sym && mode == GEMV_F32 && NR <= 2, stream_ff = sym && mode == GEMV_FF;
+  const double mbytes = (mode == GEMV_FF ? 2.0 : 1.0) * (stream || stream_ff ? 2.0 * n * (n + 1.0) : 4.0 * n * n);
   ProfScope prof(mode == GEMV_FF ? "gemv_r32_ff" : "gemv_r32_f32", mbytes + 32.0 * n * NR, 4.0 * n * n * NR, s);
   if (stream) return gemv_stream_r32<NR <= 1 ? 1 : 2>(Mhi, ld, n, w, s);
+  if (stream_ff) return gemv_stream_r32_ff(Mhi, Mlo, ld, n, NR, w, s);
   if (mode == GEMV_FF) {
     auto k = gemv_r32_kernel<NR, true>;
     const int grid = (int)gemv_grid(k, units, w);
@@ -1477,6 +1480,7 @@ cudaError_t dense_inverse_block_cg(const int32_t* ptr, const int32_t* col, const
       bcg_store_kernel<<<grid, BCG_THREADS, 0, s>>>(n, w, c0, ld, Xres, sums, project, Xhi, Xlo);
     if ((err = cudaGetLastError()) != cudaSuccess) return fail(err);
   }
+  if (!(Xd && project) && (err = symmetrize_planes(Xhi, Xlo, n, ld, s)) != cudaSuccess) return fail(err);
   if ((err = cudaStreamSynchronize(s)) != cudaSuccess) return fail(err);
   *iters = worst_iters;
   return fail(cudaSuccess);

@@ -287,8 +287,10 @@ template <int NR>
 cudaError_t gemv_stream_c64(const float2* M, int ld, int n, bool conj, GemvScratch& w, cudaStream_t s);
 template <int NR>
 cudaError_t gemv_stream_r32(const float* M, int ld, int n, GemvScratch& w, cudaStream_t s);
-// Float-float streaming GEMV of one column of a complex64 M (x split in w.xh + w.xl).
-cudaError_t gemv_stream_c64_ff(const float2* M, int ld, int n, bool conj, GemvScratch& w, cudaStream_t s);
+// Float-float streaming GEMV of nr columns of a symmetric complex64 M, or FP32 hi + lo one (x split in
+// w.xh + w.xl).
+cudaError_t gemv_stream_c64_ff(const float2* M, int ld, int n, int nr, bool conj, GemvScratch& w, cudaStream_t s);
+cudaError_t gemv_stream_r32_ff(const float* hi, const float* lo, int ld, int n, int nr, GemvScratch& w, cudaStream_t s);
 int padded_ld(int n);
 
 // Device memory from the device's stream-ordered pool, which keeps freed memory mapped: the
@@ -448,13 +450,15 @@ int build_amg(const std::vector<int32_t>& ptr, const std::vector<int32_t>& col, 
 // Dense inverse of a sparse SPD matrix (or of the singular cell Laplacian restricted to 1^perp,
 // with project = true: columns e_c - 1/n, result with zero column means = the pseudo-inverse),
 // by block CG, preconditioned by one multigrid V(1,1) cycle when H is given.  A in CSR (device,
-// n x n, FP64); output in FP32 hi + lo planes (n rows, padded_ld(n) stride).  Work buffers are
+// n x n, FP64); output in FP32 hi + lo planes (n rows, padded_ld(n) stride), exactly symmetric.  Work buffers are
 // allocated inside.  *iters receives the iteration count of the slowest column block.
 // With Xd (and project), the result goes to Xd (FP64, n rows, padded_ld(n) stride) as
 // X - colmean + 1/n, an approximation of (L + 1 1^T / n)^{-1}, instead of the FP32 planes.
 cudaError_t dense_inverse_block_cg(const int32_t* ptr, const int32_t* col, const double* val, int n, bool project,
                                    const AmgHierarchy* H, double tol, int max_iter, float* Xhi, float* Xlo,
                                    int* iters, cudaStream_t s, double* Xd = nullptr);
+// hi + lo <- its symmetric part, in place (k_factor.cu)
+cudaError_t symmetrize_planes(float* hi, float* lo, int n, int ld, cudaStream_t s);
 // Newton-Schulz refinement of X ~ M^{-1} (k_factor.cu) for M = L + 1 1^T / n (project: writes
 // (Sigma^T Sigma)^+ = sym(X) - 1 1^T / n) or M = L (writes sym(X)) to the FP32 hi + lo planes.  lap: L
 // as a graph Laplacian, or null: per row three neighbours, n where there is none, and the diagonal entry
