@@ -512,7 +512,7 @@ int ensure_workspace(rfcmp_op* op, int cols) {
     }
     if (bf) {
       RF_TRY(dalloc(&ws->ms.xb, (size_t)4 * cols * ws->ms.cap_ld, ws->owned));
-      RF_TRY(dalloc(&ws->ms.D, (size_t)4 * cols * capn, ws->owned));
+      RF_TRY(dalloc(&ws->ms.D, (size_t)4 * cols * capn + (size_t)(GEMM_SLOTS + 1) * 256 * std::min(cols, 64), ws->owned));
     }
     if (ex) {
       RF_TRY(dalloc(&ws->ms.xd, (size_t)EXACT_DIGITS * 2 * cols * ws->ms.cap_ld, ws->owned));

@@ -51,6 +51,7 @@ struct GemmMaps {
   CUtensorMap b[2][2];
 };
 
+constexpr int GEMM_SHARE = 4;  // fewest K blocks of a split share
 constexpr int GEMM_THREADS = 192;  // warp 0 loads, warp 1 issues MMAs, warps 2-5 drain accumulators
 
 // Output tile of linear index lin: groups of GROUP_M row tiles, the row tile fastest within a
@@ -99,7 +100,29 @@ __device__ __forceinline__ void seq_tile(int i, int tm, int tn, int upper, int& 
   else tile_of(i, tm, tn, tile_m, tile_n);
 }
 
-// Persistent kernel: CTA b takes the tiles b, b + G, b + 2G, ... (G CTAs, one per SM).  The
+// Work of CTA b of G: body(tile, q0, q1), the K blocks q0 .. q1 - 1 (of total) of an output tile, until it
+// returns false.  Whole tiles b, b + G, b + 2G, ..., or (split) an equal share of the K blocks of all tiles
+// in their order, at most one tile's end and another's start not its own.
+template <class F>
+__device__ __forceinline__ void gemm_pieces(int tiles, int total, int split, F&& body) {
+  if (split) {
+    const uint32_t T = (uint32_t)tiles * total, G = gridDim.x;
+    uint32_t u = blockIdx.x * T / G;
+    const uint32_t end = (blockIdx.x + 1) * T / G;
+    while (u < end) {
+      const uint32_t t = u / total, q0 = u - t * total, q1 = min((uint32_t)total, q0 + (end - u));
+      if (!body((int)t, (int)q0, (int)q1)) return;
+      u += q1 - q0;
+    }
+  } else {
+    for (int lin = blockIdx.x; lin < tiles; lin += gridDim.x)
+      if (!body(lin, 0, total)) return;
+  }
+}
+
+// Persistent kernel: CTA b takes the tiles b, b + G, b + 2G, ... (G CTAs, one per SM) or its share of their
+// K blocks.  Split, CTA b writes its sum of tile t to the tile slot t + b of D (b and t only grow along the
+// sequence, so slots are distinct) and the reader adds a tile's slots.  The
 // producer keeps the stage ring full across tile boundaries; the MMA warp accumulates tile t into
 // tensor-memory buffer t % 2 while the epilogue warps drain buffer (t - 1) % 2, so a tile's
 // epilogue overlaps the next tile's main loop.  The epilogue goes through a shared-memory
@@ -107,7 +130,7 @@ __device__ __forceinline__ void seq_tile(int i, int tm, int tn, int upper, int& 
 template <int BN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask, int M, int N, int K,
-                   float* __restrict__ D, long long ldd, int accumulate, int* __restrict__ err, int upper) {
+                   float* __restrict__ D, long long ldd, int accumulate, int* __restrict__ err, int upper, int split) {
   RF_COUNT_LAUNCH();
   using C = TileCfg<BN>;
   constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, TILE_B = C::TILE_B;
@@ -155,18 +178,16 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
     if (lane == 0) {
       // producer: TMA loads into the stage ring, tile after tile
       long long it = 0;
-      bool ok = true;
-      for (int lin = blockIdx.x; lin < tiles && ok; lin += gridDim.x) {
+      gemm_pieces(tiles, total, split, [&](int lin, int q0, int q1) {
         int tile_m, tile_n;
         seq_tile(lin, tm, tn, upper, tile_m, tile_n);
         const int m0 = tile_m * BM, n0 = tile_n * BN;
-        for (int q = 0; q < total; ++q, ++it) {
+        for (int q = q0; q < q1; ++q, ++it) {
           const int s = (int)(it % STAGES);
           const long long round = it / STAGES;
           if (round > 0 && !mbar_wait(&empty[s], (uint32_t)((round - 1) & 1))) {
             atomicExch(err, 1);
-            ok = false;
-            break;
+            return false;
           }
           uint8_t* st = smem + s * STAGE_BYTES;
           const int seg = q / kblocks, kx = (q % kblocks) * BK;
@@ -176,7 +197,8 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
           tma_load_2d(st + 2 * TILE_A, &maps.b[seg][0], &full[s], kx, n0);
           tma_load_2d(st + 2 * TILE_A + TILE_B, &maps.b[seg][1], &full[s], kx, n0);
         }
-      }
+        return true;
+      });
       // the copies of the last rounds have landed before the CTA may exit (bounded)
       for (long long j = it - 1; j >= 0 && j >= it - STAGES; --j)
         if (!mbar_wait(&full[j % STAGES], (uint32_t)((j / STAGES) & 1))) atomicExch(err, 4);
@@ -187,24 +209,20 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
       const uint32_t id_pos = idesc_bf16(BM, BN, false), id_neg = idesc_bf16(BM, BN, true);
       long long it = 0;
       int t = 0;  // tiles of this CTA so far
-      bool ok = true;
-      for (int lin = blockIdx.x; lin < tiles && ok; lin += gridDim.x) {
-        int tile_m, tile_n;
-        seq_tile(lin, tm, tn, upper, tile_m, tile_n);
+      gemm_pieces(tiles, total, split, [&](int, int q0, int q1) {
         const int b = t & 1, use = t >> 1;
         if (use > 0 && !mbar_wait(&acc_empty[b], (uint32_t)((use - 1) & 1))) {
           atomicExch(err, 5);
-          break;
+          return false;
         }
         tc_fence_after();
         const uint32_t acc = tmem + (uint32_t)b * ACC_COLS;
-        for (int q = 0; q < total; ++q, ++it) {
+        for (int q = q0; q < q1; ++q, ++it) {
           const int s = (int)(it % STAGES);
           const long long round = it / STAGES;
           if (!mbar_wait(&full[s], (uint32_t)(round & 1))) {
             atomicExch(err, 2);
-            ok = false;
-            break;
+            return false;
           }
           tc_fence_after();
           const int seg = q / kblocks;
@@ -216,16 +234,16 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
             const uint32_t off = kk * 32;  // 16 BF16 along K inside the 128-byte swizzled row
             const uint64_t ah = sw128_desc(a_hi + off), al = sw128_desc(a_lo + off);
             const uint64_t bh = sw128_desc(b_hi + off), bl = sw128_desc(b_lo + off);
-            mma_bf16(acc, ah, bh, idesc, (q > 0 || kk > 0) ? 1u : 0u);
+            mma_bf16(acc, ah, bh, idesc, (q > q0 || kk > 0) ? 1u : 0u);
             mma_bf16(acc, ah, bl, idesc, 1u);
             mma_bf16(acc, al, bh, idesc, 1u);
           }
           mma_commit(&empty[s]);  // the stage is free once these MMAs have read it
         }
-        if (!ok) break;
         mma_commit(&acc_full[b]);  // arrives when the tile's MMAs have completed
         ++t;
-      }
+        return true;
+      });
       // every MMA issued above has completed before tensor memory is released (bounded)
       mma_commit(drained);
       if (!mbar_wait(drained, 0)) atomicExch(err, 6);
@@ -235,17 +253,18 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
     const int quarter = warp & 3;
     float* tb = epi + (warp - 2) * 32 * 33;
     int t = 0;
-    for (int lin = blockIdx.x; lin < tiles; lin += gridDim.x) {
+    gemm_pieces(tiles, total, split, [&](int lin, int, int) {
       int tile_m, tile_n;
       seq_tile(lin, tm, tn, upper, tile_m, tile_n);
       const int b = t & 1, use = t >> 1;
       const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (uint32_t)(use & 1)));
       if (!ok) {
         if (lane == 0) atomicExch(err, 3);
-        break;
+        return false;
       }
       tc_fence_after();
       const int r0 = tile_m * BM + 32 * quarter, n0 = tile_n * BN;
+      const int d0 = (split ? lin + (int)blockIdx.x : tile_m) * BM + 32 * quarter;  // row of D
 #pragma unroll 1
       for (int c0 = 0; c0 < BN; c0 += 32) {
         uint32_t r[32];
@@ -258,9 +277,8 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
         if (col < N) {
 #pragma unroll 4
           for (int i = 0; i < 32; ++i) {
-            const int row = r0 + i;
-            if (row >= M) break;
-            float* dst = D + (size_t)row * ldd + col;
+            if (r0 + i >= M) break;
+            float* dst = D + (size_t)(d0 + i) * ldd + col;
             float v = tb[i * 33 + lane];
             if (accumulate) v += *dst;
             *dst = v;
@@ -272,7 +290,8 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
       tc_fence_before();
       if (lane == 0) mbar_arrive(&acc_empty[b]);
       ++t;
-    }
+      return true;
+    });
   }
   __syncwarp();
   tc_fence_before();
@@ -302,7 +321,8 @@ __global__ void split_bf16_kernel(const T* __restrict__ src, long long ld_src, i
 
 template <int BN>
 cudaError_t gemm_launch(const SplitOperand* A, const SplitOperand* B, const int* negate, int nseg, int M, int N, int K,
-                        float* D, long long ldd, bool accumulate, int* err_dev, cudaStream_t s, bool upper) {
+                        float* D, long long ldd, bool accumulate, int* err_dev, cudaStream_t s, bool upper,
+                        GemmSplit* split) {
   if (upper && BN != BM) return cudaErrorInvalidValue;
   using C = TileCfg<BN>;
   GemmMaps maps;
@@ -336,7 +356,19 @@ cudaError_t gemm_launch(const SplitOperand* A, const SplitOperand* B, const int*
     if (sms_err == cudaSuccess) sms_err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   });
   if (sms_err != cudaSuccess || sms <= 0) return sms_err != cudaSuccess ? sms_err : cudaErrorInvalidValue;
-  const int grid = (int)std::max(1LL, std::min<long long>(tiles, sms));
+  int grid = (int)std::max(1LL, std::min<long long>(tiles, sms));
+  if (split) {
+    // One column tile only: with several, CTAs that work on one panel of A at the same K blocks share it in L2.
+    // A share is at least GEMM_SHARE K blocks; fewer do not pay for a CTA's start.
+    const long long total = (long long)nseg * ((K + BK - 1) / BK), T = tiles * total;
+    const int g = (int)std::min<long long>(std::min(sms, GEMM_SLOTS), std::max(tiles, T / GEMM_SHARE));
+    split->ctas = 0;
+    if (tnl == 1 && !accumulate && T * g < 0x7fffffffLL && tiles % g != 0) {
+      grid = split->ctas = g;
+      split->tiles = (int)tiles;
+      split->total = (int)total;
+    }
+  }
   double frac = 1.0;  // share of the output tiles computed
   if (upper) {
     const double tm = (M + BM - 1) / BM, tn = (N + BN - 1) / BN;
@@ -344,7 +376,7 @@ cudaError_t gemm_launch(const SplitOperand* A, const SplitOperand* B, const int*
   }
   ProfScope prof("gemm_bf16x3", 0.0, 6.0 * (double)M * N * K * nseg * frac, s);
   gemm_bf16x3_kernel<BN><<<grid, GEMM_THREADS, C::SMEM_BYTES, s>>>(maps, nseg, neg_mask, M, N, K, D, ldd,
-                                                                   accumulate ? 1 : 0, err_dev, upper ? 1 : 0);
+                                                                   accumulate ? 1 : 0, err_dev, upper ? 1 : 0, split && split->ctas);
   return cudaGetLastError();
 }
 
@@ -392,12 +424,28 @@ __global__ void split_x_kernel(const double2* __restrict__ X, int n, int nr, lon
 // Y[:, r] = scale * op(T) X[:, r] (+ Y) from D = [Tr; Ti] [Xr Xi] (2n x 2nr, row stride ldd):
 // T X = (Tr Xr - Ti Xi) + i (Tr Xi + Ti Xr); conj(T) flips the sign of the Ti terms.  With real,
 // D = P [Xr Xi] (n x 2nr) of a real P and Y = scale * (D[:, r] + i D[:, nr + r]) (+ Y).
+// P: how D was split; the sum of a tile's slots in FP64.
 // 32 x 32 tiles of (row i, column r) go through shared memory so that both the reads of D
 // (along r) and the writes of Y (along i) are coalesced.
 constexpr int CT = 32;
-__global__ void combine_cplx_kernel(const float* __restrict__ D, long long ldd, int n, int nr, int conj, int real,
-                                    double2 scale, int accumulate, double2* __restrict__ Y) {
+__global__ void combine_cplx_kernel(const float* __restrict__ D, long long ldd, GemmSplit P, int n, int nr, int conj,
+                                    int real, double2 scale, int accumulate, double2* __restrict__ Y) {
   RF_COUNT_LAUNCH();
+  auto row2 = [&](int i, int r) {  // columns r and nr + r of row i
+    if (!P.ctas) {
+      const float* d = D + (size_t)i * ldd + r;
+      return make_double2((double)d[0], (double)d[nr]);
+    }
+    const uint32_t t = (uint32_t)i / BM, T = (uint32_t)P.tiles * P.total;
+    const uint32_t b0 = ((t * P.total + 1) * P.ctas - 1) / T, b1 = ((t + 1) * P.total * P.ctas - 1) / T;
+    const float* d = D + ((size_t)(t + b0) * BM + (uint32_t)i % BM) * ldd + r;
+    double2 v = make_double2(0.0, 0.0);
+    for (uint32_t b = b0; b <= b1; ++b, d += BM * ldd) {
+      v.x += (double)d[0];
+      v.y += (double)d[nr];
+    }
+    return v;
+  };
   __shared__ double2 t[CT][CT + 1];
   const int i0 = blockIdx.x * CT, r0 = blockIdx.y * CT;
   const double sg = conj ? -1.0 : 1.0;
@@ -405,14 +453,11 @@ __global__ void combine_cplx_kernel(const float* __restrict__ D, long long ldd, 
     const int i = i0 + ii, r = r0 + threadIdx.x;
     double2 v = make_double2(0.0, 0.0);
     if (i < n && r < nr) {
-      const float* top = D + (size_t)i * ldd;
-      if (real) {
-        v.x = (double)top[r];
-        v.y = (double)top[nr + r];
-      } else {
-        const float* bot = D + (size_t)(n + i) * ldd;
-        v.x = (double)top[r] - sg * (double)bot[nr + r];
-        v.y = (double)top[nr + r] + sg * (double)bot[r];
+      v = row2(i, r);
+      if (!real) {
+        const double2 bot = row2(n + i, r);
+        v.x -= sg * bot.y;
+        v.y += sg * bot.x;
       }
     }
     t[ii][threadIdx.x] = v;
@@ -455,11 +500,13 @@ cudaError_t cplx_gemm(const CplxPlanes& T, const double2* X, double2* Y, int nr,
   SplitOperand A, B;
   A.hi = T.rh; A.lo = T.rl; A.rows = 2 * n; A.ld = ldp;
   B.hi = bh; B.lo = bl; B.rows = 2 * nr; B.ld = ldp;
+  GemmSplit P;
   cudaError_t e;
-  if ((e = gemm_bf16x3(&A, &B, nullptr, 1, 2 * n, 2 * nr, n, w.D, 2 * nr, false, w.err, s, w.bn)) != cudaSuccess)
+  if ((e = gemm_bf16x3(&A, &B, nullptr, 1, 2 * n, 2 * nr, n, w.D, 2 * nr, false, w.err, s, w.bn, false, &P)) !=
+      cudaSuccess)
     return e;
   dim3 g2((n + CT - 1) / CT, (nr + CT - 1) / CT), b2(CT, 8);
-  combine_cplx_kernel<<<g2, b2, 0, s>>>(w.D, 2 * nr, n, nr, conj ? 1 : 0, 0, scale, accumulate ? 1 : 0, Y);
+  combine_cplx_kernel<<<g2, b2, 0, s>>>(w.D, 2 * nr, P, n, nr, conj ? 1 : 0, 0, scale, accumulate ? 1 : 0, Y);
   return cudaGetLastError();
 }
 
@@ -476,10 +523,13 @@ cudaError_t real_gemm(const RealPlanes& P, const double2* X, double2* Y, int nr,
   SplitOperand A, B;
   A.hi = P.h; A.lo = P.l; A.rows = n; A.ld = ldp;
   B.hi = bh; B.lo = bl; B.rows = 2 * nr; B.ld = ldp;
+  GemmSplit split;
   cudaError_t e;
-  if ((e = gemm_bf16x3(&A, &B, nullptr, 1, n, 2 * nr, n, w.D, 2 * nr, false, w.err, s, w.bn)) != cudaSuccess) return e;
+  if ((e = gemm_bf16x3(&A, &B, nullptr, 1, n, 2 * nr, n, w.D, 2 * nr, false, w.err, s, w.bn, false, &split)) !=
+      cudaSuccess)
+    return e;
   dim3 g2((n + CT - 1) / CT, (nr + CT - 1) / CT), b2(CT, 8);
-  combine_cplx_kernel<<<g2, b2, 0, s>>>(w.D, 2 * nr, n, nr, 0, 1, make_double2(scale, 0.0), accumulate ? 1 : 0, Y);
+  combine_cplx_kernel<<<g2, b2, 0, s>>>(w.D, 2 * nr, split, n, nr, 0, 1, make_double2(scale, 0.0), accumulate ? 1 : 0, Y);
   return cudaGetLastError();
 }
 
@@ -499,17 +549,17 @@ cudaError_t split_bf16_f64(const double* src, long long ld_src, int rows, int co
 
 cudaError_t gemm_bf16x3(const SplitOperand* A, const SplitOperand* B, const int* negate, int nseg, int M, int N,
                         int K, float* D, long long ldd, bool accumulate, int* err_dev, cudaStream_t s, int bn,
-                        bool upper) {
+                        bool upper, GemmSplit* split) {
   if (nseg < 1 || nseg > 2 || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
   if (upper) bn = 128;
   if (bn == 0) bn = N <= 32 ? 32 : (N <= 64 ? 64 : 128);
   switch (bn) {
     case 32:
-      return gemm_launch<32>(A, B, negate, nseg, M, N, K, D, ldd, accumulate, err_dev, s, upper);
+      return gemm_launch<32>(A, B, negate, nseg, M, N, K, D, ldd, accumulate, err_dev, s, upper, split);
     case 64:
-      return gemm_launch<64>(A, B, negate, nseg, M, N, K, D, ldd, accumulate, err_dev, s, upper);
+      return gemm_launch<64>(A, B, negate, nseg, M, N, K, D, ldd, accumulate, err_dev, s, upper, split);
     case 128:
-      return gemm_launch<128>(A, B, negate, nseg, M, N, K, D, ldd, accumulate, err_dev, s, upper);
+      return gemm_launch<128>(A, B, negate, nseg, M, N, K, D, ldd, accumulate, err_dev, s, upper, split);
     default:
       return cudaErrorInvalidValue;
   }

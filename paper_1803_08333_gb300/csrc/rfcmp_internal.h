@@ -198,9 +198,16 @@ struct SplitOperand {
 // bounded device-side wait gave up.
 // bn selects the N tile (32, 64 or 128); 0 picks it from N.  With upper, only the 128 x 128 tiles
 // on or above the diagonal are computed (for a result known to be symmetric).
+// With split (N within one tile): the K blocks of all row tiles may be dealt to the CTAs in equal shares, which
+// writes *split with ctas > 0 and D as tile slots of 128 rows (GEMM_SLOTS more than the tiles), the sum of
+// a tile by CTA b in slot tile + b.
+constexpr int GEMM_SLOTS = 160;  // bound on the CTAs of a split product
+struct GemmSplit {
+  int ctas = 0, tiles = 0, total = 0;  // total: K blocks of a tile
+};
 cudaError_t gemm_bf16x3(const SplitOperand* A, const SplitOperand* B, const int* negate, int nseg, int M, int N,
                         int K, float* D, long long ldd, bool accumulate, int* err_dev, cudaStream_t s, int bn = 0,
-                        bool upper = false);
+                        bool upper = false, GemmSplit* split = nullptr);
 cudaError_t split_bf16_f32(const float* src, long long ld_src, int rows, int cols, __nv_bfloat16* hi,
                            __nv_bfloat16* lo, long long ld_dst, cudaStream_t s);
 
@@ -219,7 +226,7 @@ struct RealPlanes {  // real n x n: hi/lo, row stride ldp
 // products (2 x cap_n x cap_cols); err receives device-side timeout codes.
 struct MrhsScratch {
   __nv_bfloat16* xb = nullptr;
-  float* D = nullptr;  // 4 x cap_cols x cap_n
+  float* D = nullptr;  // 4 x cap_cols x cap_n, and GEMM_SLOTS + 1 tiles of 128 rows of at most 128 columns
   int* err = nullptr;
   int cap_cols = 0, cap_n = 0;
   long long cap_ld = 0;
