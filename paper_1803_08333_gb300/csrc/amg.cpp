@@ -221,7 +221,26 @@ int build_amg(const std::vector<int32_t>& ptr, const std::vector<int32_t>& col, 
       P.ptr[i + 1] = (int32_t)P.col.size();
     }
     Csr R = transpose(P);
-    Csr Ac = multiply(R, multiply(A, P));
+    Csr AP = multiply(A, P);
+    Csr Ac = multiply(R, AP);
+    // S = (I - w D^{-1} A) P by merging the sorted rows of P and A P
+    L.S_ptr.assign(A.n + 1, 0);
+    L.S_colsum.assign(na, 0.0);
+    for (int i = 0; i < A.n; ++i) {
+      int p = P.ptr[i], q = AP.ptr[i];
+      const double f = L.omega / L.diag[i];
+      while (p < P.ptr[i + 1] || q < AP.ptr[i + 1]) {
+        const int cp = p < P.ptr[i + 1] ? P.col[p] : na, cq = q < AP.ptr[i + 1] ? AP.col[q] : na;
+        const int c = std::min(cp, cq);
+        double v = 0.0;
+        if (cp == c) v += P.val[p++];
+        if (cq == c) v -= f * AP.val[q++];
+        L.S_col.push_back(c);
+        L.S_val.push_back(v);
+        L.S_colsum[c] += v;
+      }
+      L.S_ptr[i + 1] = (int32_t)L.S_col.size();
+    }
     L.A_ptr = A.ptr;
     L.A_col = A.col;
     L.A_val = A.val;

@@ -1389,12 +1389,15 @@ int build_factor(const std::vector<int32_t>& ptr, const std::vector<int32_t>& co
     double res = 1.0;
     for (int attempt = 0; attempt < 2 && err == cudaSuccess && !(res <= accept); ++attempt) {
       int it = 0;
-      err = dense_inverse_block_cg(dptr, dcol, dval, n, project, &H, NS_START_TOL, attempt == 0 ? 0 : 20000, f->hi,
-                                   f->lo, &it, 0, Xd);
+      bool start = false;
+      if (attempt == 0) err = multigrid_inverse(H, n, Xd, padded_ld(n), &start, 0);
+      if (err == cudaSuccess && !start)
+        err = dense_inverse_block_cg(dptr, dcol, dval, n, project, &H, NS_START_TOL, attempt == 0 ? 0 : 20000, f->hi,
+                                     f->lo, &it, 0, Xd);
       iters += it;
       int st = 0;
       if (err == cudaSuccess)
-        err = newton_schulz_pseudo_inverse(dptr, dcol, dval, dlap, n, true, Xd, padded_ld(n), NS_MAX_STEPS, target, f->hi,
+        err = newton_schulz_pseudo_inverse(dptr, dcol, dval, dlap, n, true, start, Xd, padded_ld(n), NS_MAX_STEPS, target, f->hi,
                                            f->lo, &st, &res, 0);
       steps += st;
     }
@@ -1421,7 +1424,7 @@ int build_factor(const std::vector<int32_t>& ptr, const std::vector<int32_t>& co
     double res = 1.0;
     if (err == cudaSuccess) err = jacobi_start(dptr, dcol, dval, n, jacobi_c, Xd, padded_ld(n), 0);
     if (err == cudaSuccess)
-      err = newton_schulz_pseudo_inverse(dptr, dcol, dval, nullptr, n, false, Xd, padded_ld(n), NS_MAX_STEPS, target, f->hi,
+      err = newton_schulz_pseudo_inverse(dptr, dcol, dval, nullptr, n, false, true, Xd, padded_ld(n), NS_MAX_STEPS, target, f->hi,
                                          f->lo, &steps, &res, 0);
     if (Xd) dev_free(Xd);
     f->ns_steps = steps;

@@ -445,6 +445,8 @@ struct AmgLevelHost {
   std::vector<double> diag;
   std::vector<int32_t> A_ptr, A_col, P_ptr, P_col, R_ptr, R_col;  // A (n x n), P (n x nc), R = P^T
   std::vector<double> A_val, P_val, R_val;
+  std::vector<int32_t> S_ptr, S_col;  // S = (I - w D^{-1} A) P, the prolongation and one smoothing step (n x nc)
+  std::vector<double> S_val, S_colsum;
 };
 struct AmgHierarchy {
   std::vector<AmgLevelHost> levels;
@@ -464,6 +466,10 @@ int build_amg(const std::vector<int32_t>& ptr, const std::vector<int32_t>& col, 
 cudaError_t dense_inverse_block_cg(const int32_t* ptr, const int32_t* col, const double* val, int n, bool project,
                                    const AmgHierarchy* H, double tol, int max_iter, float* Xhi, float* Xlo,
                                    int* iters, cudaStream_t s, double* Xd = nullptr);
+// X (n rows, stride ld) <- (I - J) M (I - J) + J, J = 1 1^T / n, M one V(1,1) cycle of H: an approximation of
+// (L + J)^{-1}, exactly symmetric (k_factor.cu).  *done = false, nothing queued, where the hierarchy has no
+// levels or a coarse row does not fit in shared memory.
+cudaError_t multigrid_inverse(const AmgHierarchy& H, int n, double* X, long long ld, bool* done, cudaStream_t s);
 // hi + lo <- its symmetric part, in place (k_factor.cu)
 cudaError_t symmetrize_planes(float* hi, float* lo, int n, int ld, cudaStream_t s);
 // Newton-Schulz refinement of X ~ M^{-1} (k_factor.cu) for M = L + 1 1^T / n (project: writes
@@ -471,7 +477,7 @@ cudaError_t symmetrize_planes(float* hi, float* lo, int n, int ld, cudaStream_t 
 // as a graph Laplacian, or null: per row three neighbours, n where there is none, and the diagonal entry
 // (16 bits each, two rows a word; an odd n's last row is empty).
 cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col, const double* val, const uint4* lap,
-                                         int n, bool project, double* X, long long ldx, int max_steps, double tol, float* Xhi,
+                                         int n, bool project, bool symmetric, double* X, long long ldx, int max_steps, double tol, float* Xhi,
                                          float* Xlo, int* steps_done, double* final_residual, cudaStream_t s);
 // X = c D^{-1} for the diagonal D of a CSR matrix (n x n, row stride ldx; the rest of X zeroed)
 cudaError_t jacobi_start(const int32_t* ptr, const int32_t* col, const double* val, int n, double c, double* X,
