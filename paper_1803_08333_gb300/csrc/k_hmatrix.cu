@@ -12,6 +12,7 @@
 // resident dense matrix (rows and columns gathered through the cluster permutation), blocks whose
 // crosses reach the rank cap, or would take at least the block's own entries, stay dense, and the factors and dense blocks are packed into one
 // buffer per matrix.  The product y = H x (FP64 accumulation) runs over cross items and row tiles.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -32,6 +33,8 @@
 #include "rfcmp_internal.h"
 
 namespace rfcmp {
+
+namespace cg = cooperative_groups;
 
 RF_LAUNCH_READER(launches_hmatrix)
 
@@ -486,10 +489,10 @@ __global__ void __launch_bounds__(HM_THREADS)
 //   hm_gather   x into cluster order, the columns of a group interleaved
 //   hm_cross    t = Vt x[c0..c1) and t' = U x[r0..r1) of every low-rank block, one warp per four
 //               crosses of one side, so an x entry is read once for four crosses
-//   hm_rows     y of one tile of at most 32 rows per CTA: every block that covers the tile adds U t
+//   hm_rows     y of one tile of at most 32 rows per CTA or cluster of CTAs: every block that covers the tile adds U t
 //               (or Vt^T t' below the diagonal, or its dense entries), lane = row, the blocks dealt to
-//               the CTA's warps; one store per row through the permutation
-// Every stored entry is used once per side, so no sum crosses a CTA: no atomics, no zeroed output,
+//               its warps; one store per row through the permutation
+// Every stored entry is used once per side, so no sum crosses a cluster: no atomics, no zeroed output,
 // and a product is the same bits on every run.  Bound: the FP64 pipe (2 lanes per clock and SM, 90 to
 // 93 % busy), 8 multiply-adds per stored entry and column; the FP32 entries are widened with integer
 // operations, which keeps the conversions off that pipe.  Measured on GB300: both products of an
@@ -586,14 +589,14 @@ __device__ __forceinline__ void madd(double (&acc)[2 * HM_COLS], float2 e, const
   }
 }
 
-// the sums of one row (row0 + lane) of a tile over the cover entries begin + w, begin + w + 8, ...
+// the sums of one row (row0 + lane) of a tile over the cover entries begin + w, begin + w + step, ...
 template <int NC>
 __device__ __forceinline__ void tile_rows(const HmTile& T, const int32_t* __restrict__ cover,
                                           const HmBlockDev* __restrict__ blk, const float2* __restrict__ H,
                                           const double2* __restrict__ xg, const double2* __restrict__ t, int nrhs,
-                                          int w, int lane, double (&acc)[2 * HM_COLS]) {
+                                          int w, int step, int lane, double (&acc)[2 * HM_COLS]) {
   const bool live = lane < T.rows;
-  for (int q = T.begin + w; q < T.end; q += HM_ROW_WARPS) {
+  for (int q = T.begin + w; q < T.end; q += step) {
     const int code = cover[q];
     const HmBlockDev B = blk[code >> 1];
     const int cols = code & 1, m = B.r1 - B.r0, nn = B.c1 - B.c0;
@@ -621,6 +624,7 @@ __device__ __forceinline__ void tile_rows(const HmTile& T, const int32_t* __rest
   }
 }
 
+// A cluster of CTAs per tile and group, the cover entries dealt to all their warps; the first adds their sums in order.
 __global__ void __launch_bounds__(HM_THREADS)
     hm_rows_kernel(const HmTile* __restrict__ tiles, const int32_t* __restrict__ cover,
                    const HmBlockDev* __restrict__ blk, const float2* __restrict__ H, const double2* __restrict__ xp,
@@ -628,29 +632,52 @@ __global__ void __launch_bounds__(HM_THREADS)
                    int nrhs) {
   RF_COUNT_LAUNCH();
   __shared__ double part[HM_ROW_WARPS][2 * HM_COLS][HM_TILE];
-  const HmTile T = tiles[blockIdx.x];
+  __shared__ double sums[HM_THREADS];
+  const cg::cluster_group cl = cg::this_cluster();
+  const int team = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const HmTile T = tiles[blockIdx.x / team];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = blockIdx.y * HM_COLS, nc = min(HM_COLS, nrhs - g);
   const double2* xg = xp + (size_t)g * n;
+  const int first = w * team + rank, step = HM_ROW_WARPS * team;
   double acc[2 * HM_COLS];
 #pragma unroll
   for (int k = 0; k < 2 * HM_COLS; ++k) acc[k] = 0.0;
   switch (nc) {
-    case 1: tile_rows<1>(T, cover, blk, H, xg, t + g, nrhs, w, lane, acc); break;
-    case 2: tile_rows<2>(T, cover, blk, H, xg, t + g, nrhs, w, lane, acc); break;
-    case 3: tile_rows<3>(T, cover, blk, H, xg, t + g, nrhs, w, lane, acc); break;
-    default: tile_rows<4>(T, cover, blk, H, xg, t + g, nrhs, w, lane, acc); break;
+    case 1: tile_rows<1>(T, cover, blk, H, xg, t + g, nrhs, first, step, lane, acc); break;
+    case 2: tile_rows<2>(T, cover, blk, H, xg, t + g, nrhs, first, step, lane, acc); break;
+    case 3: tile_rows<3>(T, cover, blk, H, xg, t + g, nrhs, first, step, lane, acc); break;
+    default: tile_rows<4>(T, cover, blk, H, xg, t + g, nrhs, first, step, lane, acc); break;
   }
 #pragma unroll
   for (int k = 0; k < 2 * HM_COLS; ++k) part[w][k][lane] = acc[k];
   __syncthreads();
   static_assert(HM_THREADS == 2 * HM_COLS * HM_TILE, "one thread per (value, row) of a tile");
   const int k = threadIdx.x / HM_TILE, i = threadIdx.x % HM_TILE;
-  if (i >= T.rows || k >= 2 * nc) return;
   double s = 0.0;
 #pragma unroll
   for (int v = 0; v < HM_ROW_WARPS; ++v) s += part[v][k][i];
+  if (team > 1) {
+    sums[threadIdx.x] = s;
+    cl.sync();
+    if (rank == 0)
+      for (int r = 1; r < team; ++r) s += cl.map_shared_rank(sums, r)[threadIdx.x];
+    cl.sync();  // no CTA leaves while its sums may be read
+    if (rank != 0) return;
+  }
+  if (i >= T.rows || k >= 2 * nc) return;
   reinterpret_cast<double*>(y + (size_t)(g + k / 2) * n + perm[T.row0 + i])[k & 1] = s;
+}
+
+// The FP64 pipe of an SM works on a tile as long as its CTAs are there: small matrices have fewer tiles than SMs
+// (1080 functions: about 60).  Up to 8 CTAs share a tile while there are fewer than 4 an SM: 1080 functions and 720
+// cells, both products of one and of four columns 128 and 302 us with one CTA a tile, 77 and 151 so; 18000
+// functions and 12000 cells, one column 1.09 and 1.03 ms.  Cutting the entries into pieces of 16 or 32 terms as
+// well gave nothing.
+int hm_team(long long ctas) {
+  int team = 1;
+  while (team < 8 && ctas * team < 4 * 152) team *= 2;
+  return team;
 }
 
 }  // namespace
@@ -1085,6 +1112,7 @@ int rfcmp_hm_apply(rfcmp_hm* hm, int which, const rfcmp_c128* x, rfcmp_c128* y, 
   double2* xp = nullptr;
   HM_CUDA(cudaMallocAsync(&xp, (16 * (size_t)P.n + per_col) * (size_t)width, st));
   double2* t = xp + (size_t)P.n * width;
+  cudaError_t launched = cudaSuccess;
   for (int64_t c = 0; c < nrhs; c += width) {
     const int nr = (int)std::min<int64_t>(width, nrhs - c);
     const long long total = (long long)P.n * nr;
@@ -1098,11 +1126,25 @@ int rfcmp_hm_apply(rfcmp_hm* hm, int which, const rfcmp_c128* x, rfcmp_c128* y, 
       hm_cross_kernel<<<dim3((P.nitems + per - 1) / per, groups), HM_CROSS_THREADS, 0, st>>>(
           P.blocks, P.items, P.nitems, P.data, xp, t, P.n, nr);
     }
-    hm_rows_kernel<<<dim3(P.ntiles, groups), HM_THREADS, 0, st>>>(P.tiles, P.cover, P.blocks, P.data, xp, t, P.perm,
-                                                                  reinterpret_cast<double2*>(y) + (size_t)c * P.n, P.n,
-                                                                  nr);
+    const int team = hm_team((long long)P.ntiles * groups);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)team;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(P.ntiles * team), groups);
+    cfg.blockDim = dim3(HM_THREADS);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    launched = cudaLaunchKernelEx(&cfg, hm_rows_kernel, (const HmTile*)P.tiles, (const int32_t*)P.cover,
+                                  (const HmBlockDev*)P.blocks, (const float2*)P.data, (const double2*)xp,
+                                  (const double2*)t, (const int32_t*)P.perm,
+                                  reinterpret_cast<double2*>(y) + (size_t)c * P.n, P.n, nr);
+    if (launched != cudaSuccess) break;
   }
   cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = launched;
   cudaFreeAsync(xp, st);
   if (e != cudaSuccess) return set_error(RFCMP_ERR_CUDA, std::string("rfcmp_hm_apply: ") + cudaGetErrorString(e));
   return RFCMP_OK;
