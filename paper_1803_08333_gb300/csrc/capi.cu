@@ -1902,7 +1902,7 @@ int rfcmp_op_export(const rfcmp_op* op, int which, void* dst, uint64_t dst_bytes
     const int ld = which == 0 ? op->ldN : op->ldC;
     if (dst_bytes < (uint64_t)n * n * 8) return set_error(RFCMP_ERR_INVALID_ARG, "destination too small");
     const float2* M = which == 0 ? op->TA : op->V;
-    RF_CUDA(cudaMemcpy2DAsync(dst, (size_t)n * 8, M, (size_t)ld * 8, (size_t)n * 8, n, cudaMemcpyDeviceToDevice, st));
+    RF_K(copy_rows(dst, M, (size_t)ld * 8, (size_t)n * 8, n, st));
     return RFCMP_OK;
   }
   if (which == 4 && !op->gtp) return set_error(RFCMP_ERR_INVALID_ARG, "op has no G_l~p factor");
@@ -1913,9 +1913,8 @@ int rfcmp_op_export(const rfcmp_op* op, int which, void* dst, uint64_t dst_bytes
     // hi and lo planes side by side: first n*n floats hi, then n*n floats lo
     float* d = static_cast<float*>(dst);
     const int ld = padded_ld(n);
-    RF_CUDA(cudaMemcpy2DAsync(d, (size_t)n * 4, f.hi, (size_t)ld * 4, (size_t)n * 4, n, cudaMemcpyDeviceToDevice, st));
-    RF_CUDA(cudaMemcpy2DAsync(d + (size_t)n * n, (size_t)n * 4, f.lo, (size_t)ld * 4, (size_t)n * 4, n,
-                              cudaMemcpyDeviceToDevice, st));
+    RF_K(copy_rows(d, f.hi, (size_t)ld * 4, (size_t)n * 4, n, st));
+    RF_K(copy_rows(d + (size_t)n * n, f.lo, (size_t)ld * 4, (size_t)n * 4, n, st));
     return RFCMP_OK;
   }
   return set_error(RFCMP_ERR_INVALID_ARG, "unknown matrix id");

@@ -1486,6 +1486,56 @@ cudaError_t dense_inverse_block_cg(const int32_t* ptr, const int32_t* col, const
   return fail(cudaSuccess);
 }
 
+// ---------------------------------------------------------------- rows out of their padded stride
+// Bound: HBM, the bytes read and written.  One CTA per row, eight independent loads a thread: T_A and V of 17280 and
+// 11520 rows (3.45 GB) in 1.04 ms; strided device copies by the runtime took 3.45 ms.
+namespace {
+template <class T>
+__global__ void __launch_bounds__(256)
+copy_rows_kernel(T* __restrict__ dst, const T* __restrict__ src, long long ld, int width) {
+  RF_COUNT_LAUNCH();
+  const T* s = src + (size_t)blockIdx.x * ld;
+  T* d = dst + (size_t)blockIdx.x * width;
+  constexpr int U = 8;
+  for (int c0 = threadIdx.x; c0 < width; c0 += 256 * U) {
+    T v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (c0 + 256 * u < width) v[u] = s[c0 + 256 * u];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (c0 + 256 * u < width) d[c0 + 256 * u] = v[u];
+  }
+}
+template <class T>
+cudaError_t copy_rows_as(void* dst, const void* src, size_t src_stride, size_t width, int rows, cudaStream_t s) {
+  copy_rows_kernel<T><<<rows, 256, 0, s>>>(static_cast<T*>(dst), static_cast<const T*>(src),
+                                           (long long)(src_stride / sizeof(T)), (int)(width / sizeof(T)));
+  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t copy_rows(void* dst, const void* src, size_t src_stride, size_t width, int rows, cudaStream_t s) {
+  if (rows <= 0 || width == 0) return cudaSuccess;
+  ProfScope prof("copy_rows", 2.0 * (double)width * rows, 0.0, s);
+  // memory of another device than the current one, or the host's: the runtime knows the way
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  bool here = true;
+  for (const void* p : {(const void*)dst, src}) {
+    cudaPointerAttributes at{};
+    here = here && cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev;
+  }
+  if (!here) (void)cudaGetLastError();
+  // the widest word that every row starts on (sources are padded to 256 bytes)
+  const size_t low = reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src) | src_stride | width;
+  if (here && low % 16 == 0) return copy_rows_as<float4>(dst, src, src_stride, width, rows, s);
+  if (here && low % 8 == 0) return copy_rows_as<float2>(dst, src, src_stride, width, rows, s);
+  if (here && low % 4 == 0) return copy_rows_as<float>(dst, src, src_stride, width, rows, s);
+  return cudaMemcpy2DAsync(dst, width, src, src_stride, width, rows, cudaMemcpyDeviceToDevice, s);
+}
+
 RF_LAUNCH_READER(launches_linalg)
 
 }  // namespace rfcmp

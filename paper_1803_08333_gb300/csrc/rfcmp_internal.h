@@ -311,6 +311,8 @@ cudaError_t dev_malloc(T** p, size_t bytes) {
   return dev_malloc(reinterpret_cast<void**>(p), bytes);
 }
 cudaError_t dev_free(void* p);
+// dst (rows of width bytes, one after the other) <- rows of src, src_stride bytes apart
+cudaError_t copy_rows(void* dst, const void* src, size_t src_stride, size_t width, int rows, cudaStream_t s);
 // Returns the pool's unused memory of the current device to the driver.
 void dev_pool_trim();
 
