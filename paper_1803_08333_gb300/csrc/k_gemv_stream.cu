@@ -46,6 +46,50 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                : "memory");
 }
 
+// Pairs of FP32 values in one 64-bit register: the packed operations round each half as the scalar ones do and take
+// half the issue slots (measured: 128 scalar or 64 packed operations a clock and SM).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pk(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 pk(float2 v) { return pk(v.x, v.y); }
+__device__ __forceinline__ float2 unpk(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xbf800000bf800000ull, a); }  // a - 1 b
+// i z (CONJ: -i z) of z = (re, im)
+template <bool CONJ>
+__device__ __forceinline__ f32x2 times_i(f32x2 z) {
+  const float2 v = unpk(z);
+  return CONJ ? pk(v.y, -v.x) : pk(-v.y, v.x);
+}
+// (s, e): s = a + b rounded, e the rest
+__device__ __forceinline__ f32x2 two_sum2(f32x2 a, f32x2 b, f32x2& e) {
+  const f32x2 s = add2(a, b), bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+  return s;
+}
+
 // stage and phase of a ring of N stages, advanced one unit at a time (64-bit divisions of the unit number
 // by the ring's size and by the units of a row cost a fifth of a unit's work)
 template <int N>
@@ -375,11 +419,13 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // streaming layout: x is split into FP32 hi + lo, every product m * x_hi is exact as (p, e) by an
 // FMA residual, p enters a float-float (hi, lo) accumulator by an error-free two-sum and
 // e + m * x_lo its low word (about 1e-14 of sum |terms|).
-// Two CTAs per SM, two stages of 40 KB each (8 rows x 512 entries and x hi and lo of the segment): half
-// the segment with four stages took 2.28 ms where this takes 1.72 (N = 30720).
+// Bound: the FP32 pipe, 22 packed operations an entry (its real and its imaginary part times both parts of x).
+// Two CTAs per SM, two stages of 55 KB each (8 rows x 704 entries and x hi and lo of the segment), the longest
+// segments that fit: N = 30720 in 1.46 ms; segments of 512 entries 1.54, three CTAs and 448 or 256 entries 1.61 and
+// 1.78; with scalar operations (twice the issue slots) and 512 entries 1.64.
 constexpr int FF_NCTA = 2;
 constexpr int FF_NST = 2;
-constexpr int FF_ROW = SBYTES_ROW;              // bytes of a row segment
+constexpr int FF_ROW = 5632;                    // bytes of a row segment
 constexpr int FF_MAT = SROWS * FF_ROW;
 constexpr int FF_STAGE = FF_MAT + 2 * FF_ROW;   // the matrix, x hi, x lo
 static_assert(FF_NCTA * (FF_NST * FF_STAGE + 256 + 1024) <= 233472, "the SM holds FF_NCTA float-float CTAs");
@@ -392,6 +438,13 @@ __device__ __forceinline__ void ff_acc(float& hi, float& lo, float a, float bh, 
   const float bb = s - hi;
   lo += ((hi - (s - bb)) + (p - bb)) + c;
   hi = s;
+}
+// both halves: hi + lo += a b with b = bh + bl
+__device__ __forceinline__ void ff_acc(f32x2& hi, f32x2& lo, f32x2 a, f32x2 bh, f32x2 bl) {
+  const f32x2 p = mul2(a, bh), c = fma2(a, bl, fma2(a, bh, neg2(p)));
+  f32x2 rest;
+  hi = two_sum2(hi, p, rest);
+  lo = add2(lo, add2(rest, c));
 }
 template <bool CONJ>
 __global__ void __launch_bounds__(STHREADS, FF_NCTA)
@@ -447,12 +500,15 @@ gemv_stream_ff_kernel(const float2* __restrict__ M, int ld, int n, const float2*
     return;
   }
 
-  float fh[2] = {0.f, 0.f}, fl[2] = {0.f, 0.f};  // (re, im) float-float sums of row `warp`
+  // float-float sums of row `warp`: Re M x and Im M x, their real and imaginary parts paired
+  f32x2 rh = 0ull, rl = 0ull, ih = 0ull, il = 0ull;
   auto flush = [&](int rb) {
     const int row = rb * SROWS + warp;
-    const double re = warp_sum_d((double)fh[0] + (double)fl[0]);
-    const double im = warp_sum_d((double)fh[1] + (double)fl[1]);
-    fh[0] = fh[1] = fl[0] = fl[1] = 0.f;
+    f32x2 rest;
+    const float2 h = unpk(two_sum2(rh, times_i<CONJ>(ih), rest));
+    const float2 l = unpk(add2(add2(rl, times_i<CONJ>(il)), rest));
+    const double re = warp_sum_d((double)h.x + (double)l.x), im = warp_sum_d((double)h.y + (double)l.y);
+    rh = rl = ih = il = 0ull;
     if (lane == 0 && row < n) {
       double* o = reinterpret_cast<double*>(out + row);
       atomicAdd(o, scale * re);
@@ -476,18 +532,14 @@ gemv_stream_ff_kernel(const float2* __restrict__ M, int ld, int n, const float2*
       const float4* sxl = reinterpret_cast<const float4*>(st + FF_MAT + FF_ROW);
       const float4* srow = reinterpret_cast<const float4*>(st + warp * FF_ROW);
       const int nq = min(SEG, ld - cb) / 2;  // two complex entries per float4
-#pragma unroll 2
+#pragma unroll 4
       for (int q = lane; q < nq; q += 32) {
         const float4 m = srow[q], x4 = sxh[q], l4 = sxl[q];
-        const float my = CONJ ? -m.y : m.y, mw = CONJ ? -m.w : m.w;
-        ff_acc(fh[0], fl[0], m.x, x4.x, l4.x);
-        ff_acc(fh[0], fl[0], -my, x4.y, l4.y);
-        ff_acc(fh[0], fl[0], m.z, x4.z, l4.z);
-        ff_acc(fh[0], fl[0], -mw, x4.w, l4.w);
-        ff_acc(fh[1], fl[1], m.x, x4.y, l4.y);
-        ff_acc(fh[1], fl[1], my, x4.x, l4.x);
-        ff_acc(fh[1], fl[1], m.z, x4.w, l4.w);
-        ff_acc(fh[1], fl[1], mw, x4.z, l4.z);
+        const f32x2 h0 = pk(x4.x, x4.y), h1 = pk(x4.z, x4.w), l0 = pk(l4.x, l4.y), l1 = pk(l4.z, l4.w);
+        ff_acc(rh, rl, pk(m.x, m.x), h0, l0);
+        ff_acc(ih, il, pk(m.y, m.y), h0, l0);
+        ff_acc(rh, rl, pk(m.z, m.z), h1, l1);
+        ff_acc(ih, il, pk(m.w, m.w), h1, l1);
       }
     }
     __syncwarp();
@@ -890,7 +942,7 @@ cudaError_t gemv_stream_r32(const float* M, int ld, int n, GemvScratch& w, cudaS
   return launch_sym<NR, true, false>(M, ld, n, w, s);
 }
 cudaError_t gemv_stream_c64_ff(const float2* M, int ld, int n, int nr, bool conj, GemvScratch& w, cudaStream_t s) {
-  // One complex column takes the full pass: 1.64 ms against 1.87 here at N = 30720, where neither waits for HBM
+  // One complex column takes the full pass: 1.46 ms against 1.8 here at N = 30720, where neither waits for HBM
   // (7.55 GB in 1.11 ms) and the pass over whole rows keeps no column sums.
   if (nr == 1) return conj ? launch_stream_ff<true>(M, ld, n, w, s) : launch_stream_ff<false>(M, ld, n, w, s);
   return conj ? launch_sym_ff<false, true>(M, nullptr, ld, n, nr, w, s)
