@@ -395,7 +395,8 @@ int rfcmp_op_get_plan(const rfcmp_op* op, rfcmp_plan* out);
  * Profiling counters (the paper has no counterpart; measurement support).
  * When enabled, every launch of an instrumented kernel family is bracketed by
  * CUDA events on the stream it is launched on; rfcmp_profile_read
- * synchronises the device and reports per family the launch count, the sum
+ * synchronises the device and reports per family the launch count (a launch
+ * that does two products counts as two), the sum
  * of the event durations and the algorithmic bytes and FLOPs of those
  * launches (GEMV: the matrix plus the vectors it reads and writes; far-pair
  * assembly: 49 kernel evaluations per unique pair at 54 FLOPs each).

@@ -124,11 +124,11 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 __global__ void prof_begin_kernel(int scope) { g_prof_t0[scope] = global_ns(); }
-__global__ void prof_end_kernel(int scope, int fam, double bytes, double flops) {
+__global__ void prof_end_kernel(int scope, int fam, double bytes, double flops, int products) {
   const unsigned long long t = global_ns();
   DevProfFamily& f = g_prof_dev[fam];
   atomicAdd(&f.ns, t - g_prof_t0[scope]);
-  atomicAdd(&f.launches, 1ULL);
+  atomicAdd(&f.launches, (unsigned long long)products);
   atomicAdd(&f.bytes, bytes);
   atomicAdd(&f.flops, flops);
 }
@@ -194,7 +194,8 @@ uint64_t prof_capture_key() {
 }
 
 namespace rfcmp {
-ProfScope::ProfScope(const char* family, double bytes, double flops, cudaStream_t s) : s_(s) {
+ProfScope::ProfScope(const char* family, double bytes, double flops, cudaStream_t s, int products)
+    : products_(products), s_(s) {
   if (!g_prof_on.load(std::memory_order_relaxed)) return;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
@@ -224,7 +225,7 @@ ProfScope::ProfScope(const char* family, double bytes, double flops, cudaStream_
     return;
   }
   ProfFamily& f = g_prof[idx];
-  f.launches++;
+  f.launches += products;
   f.bytes += bytes;
   f.flops += flops;
   a_ = pool_event();
@@ -242,7 +243,7 @@ ProfScope::ProfScope(const char* family, double bytes, double flops, cudaStream_
 ProfScope::~ProfScope() {
   if (slot_ < 0) return;
   if (captured_) {
-    prof_end_kernel<<<1, 1, 0, s_>>>(scope_, slot_, bytes_, flops_);
+    prof_end_kernel<<<1, 1, 0, s_>>>(scope_, slot_, bytes_, flops_, products_);
     (void)cudaGetLastError();
     return;
   }
@@ -672,6 +673,14 @@ int ensure_digits(rfcmp_op* op, cudaStream_t st) {
   return RFCMP_OK;
 }
 
+// The GEMV's scratch holds the splits of four columns: one product's, or two of at most two columns (half 0 and 1).
+GemvScratch gemv_half(rfcmp_op* op, int half) {
+  GemvScratch g = op->ws->gs;
+  g.xh += (size_t)2 * half * g.cap_ld;
+  if (g.xl) g.xl += (size_t)2 * half * g.cap_ld;
+  return g;
+}
+
 // y = scale * op(M) x (+ y) for M = T_A or V: GEMV, or the tensor-core product for wide FP32 blocks
 // (split-BF16 in the inner iterations, exact digits where float-float accuracy is asked)
 int prod_c(rfcmp_op* op, bool ta, const double2* x, double2* y, int nr, bool conj, double2 scale, bool acc,
@@ -694,7 +703,7 @@ int prod_c(rfcmp_op* op, bool ta, const double2* x, double2* y, int nr, bool con
 
 // y = scale * F x (+ y) for a dense real factor
 int prod_r(rfcmp_op* op, DenseFactor& f, const double2* x, double2* y, int nr, double scale, bool acc, GemvMode m,
-           cudaStream_t st, bool fed = false) {
+           cudaStream_t st, bool fed = false, int half = 0) {
   if (m == GEMV_FF && nr >= plan_exact(op)) {
     RF_TRY(ensure_digits(op, st));
     RF_K(exact_real_gemm(f.digits, f.n, x, y, nr, scale, acc, op->ws->ms, st));
@@ -705,7 +714,18 @@ int prod_r(rfcmp_op* op, DenseFactor& f, const double2* x, double2* y, int nr, d
     RF_K(real_gemm(f.planes, x, y, nr, scale, acc, op->ws->ms, st));
     return RFCMP_OK;
   }
-  RF_K(gemv_r32(f.hi, f.lo, f.n, x, y, nr, scale, acc, m, op->ws->gs, st, fed));
+  GemvScratch gs = gemv_half(op, half);
+  RF_K(gemv_r32(f.hi, f.lo, f.n, x, y, nr, scale, acc, m, gs, st, fed));
+  return RFCMP_OK;
+}
+
+// T_A x and V x' of nr columns in one launch, from the splits in the two halves of the scratch (gemv_pairs)
+int prod_pair(rfcmp_op* op, double2* y_ta, double2* y_v, double scale_v, int nr, bool conj, GemvMode m,
+              cudaStream_t st) {
+  const GemvScratch h0 = gemv_half(op, 0), h1 = gemv_half(op, 1);
+  const GemvPart a{op->TA, (int)op->top.ne, h0.xh, h0.xl, y_ta, 1.0};
+  const GemvPart b{op->V, (int)op->top.nc, h1.xh, h1.xl, y_v, scale_v};
+  RF_K(gemv_c64_pair(a, b, nr, conj, m, op->ws->gs, st));
   return RFCMP_OK;
 }
 
@@ -718,11 +738,12 @@ bool gemv_feedable(const rfcmp_op* op, int nr, GemvMode m) {
 }
 
 // the feed of a length-n vector whose GEMV writes y (and a second GEMV of it y2); none if !on
-GemvFeed make_feed(rfcmp_op* op, bool on, int n, GemvMode m, double2* y, double2* y2 = nullptr) {
+GemvFeed make_feed(rfcmp_op* op, bool on, int n, GemvMode m, double2* y, double2* y2 = nullptr, int half = 0) {
   GemvFeed f;
   if (!on) return f;
-  f.xh = op->ws->gs.xh;
-  f.xl = m == GEMV_FF ? op->ws->gs.xl : nullptr;
+  const GemvScratch g = gemv_half(op, half);
+  f.xh = g.xh;
+  f.xl = m == GEMV_FF ? g.xl : nullptr;
   f.ld = padded_ld(n);
   f.y = y;
   f.y2 = y2;
@@ -750,10 +771,12 @@ int apply_A(rfcmp_op* op, const double2* x, double2* out, int nr, GemvMode m, cu
   const int N = (int)op->top.ne, C = (int)op->top.nc, NV = (int)op->top.nv;
   // every sparse kernel below writes the split of its output for the GEMV that reads it next
   const bool fd = gemv_feedable(op, nr, m);
+  // the products with V wait for those with T_A, to share their launch
+  const bool pair = fd && gemv_pairs(nr, m, W.gs);
   // s = Sigma^T x, z = L^+ s ; w = V Sigma^T x / (k b) (the same split of s)
-  RF_K(sigma_t(g, x, W.s, nr, st, make_feed(op, fd, C, m, W.z, W.w)));
-  RF_TRY(prod_r(op, *op->lplus, W.s, W.z, nr, 1.0, false, m, st, fd));
-  RF_TRY(prod_c(op, false, W.s, W.w, nr, false, c2(1.0 / (k * b), 0.0), false, m, st, fd));
+  RF_K(sigma_t(g, x, W.s, nr, st, make_feed(op, fd, C, m, W.z, W.w, pair)));
+  RF_TRY(prod_r(op, *op->lplus, W.s, W.z, nr, 1.0, false, m, st, fd, pair));
+  if (!pair) RF_TRY(prod_c(op, false, W.s, W.w, nr, false, c2(1.0 / (k * b), 0.0), false, m, st, fd));
   // v = (ik/a) x - (ik/a + k/b) Sigma z      = i k x_L / a - k x_S / b ; u = T_A v
   {
     EdgeCombo c;
@@ -763,7 +786,8 @@ int apply_A(rfcmp_op* op, const double2* x, double2* out, int nr, GemvMode m, cu
     c.b = c2(-k / b, -k / a);
     RF_K(edge_combo(g, c, W.v, nr, st, make_feed(op, fd, N, m, W.u)));
   }
-  RF_TRY(prod_c(op, true, W.v, W.u, nr, false, c2(1.0, 0.0), false, m, st, fd));
+  if (pair) RF_TRY(prod_pair(op, W.u, W.w, 1.0 / (k * b), nr, false, m, st));
+  else RF_TRY(prod_c(op, true, W.v, W.u, nr, false, c2(1.0, 0.0), false, m, st, fd));
   // zu = L^+ Sigma^T u ; tg = G_ll^{-1} Lambda^T u
   RF_K(sigma_t(g, W.u, W.s, nr, st, make_feed(op, fd, C, m, W.zu)));
   RF_TRY(prod_r(op, *op->lplus, W.s, W.zu, nr, 1.0, false, m, st, fd));
@@ -786,9 +810,10 @@ int apply_A(rfcmp_op* op, const double2* x, double2* out, int nr, GemvMode m, cu
     RF_K(edge_combo(g, c, W.y, nr, st, make_feed(op, fd, N, m, W.up)));
   }
   // up = conj(T_A) y ; vp = conj(V) (Sigma^T Sigma) q / (k b)
-  RF_TRY(prod_c(op, true, W.y, W.up, nr, true, c2(1.0, 0.0), false, m, st, fd));
-  RF_K(lap_apply(g, W.q, W.Lq, nr, st, make_feed(op, fd, C, m, W.vp)));
-  RF_TRY(prod_c(op, false, W.Lq, W.vp, nr, true, c2(1.0 / (k * b), 0.0), false, m, st, fd));
+  if (!pair) RF_TRY(prod_c(op, true, W.y, W.up, nr, true, c2(1.0, 0.0), false, m, st, fd));
+  RF_K(lap_apply(g, W.q, W.Lq, nr, st, make_feed(op, fd, C, m, W.vp, nullptr, pair)));
+  if (pair) RF_TRY(prod_pair(op, W.up, W.vp, 1.0 / (k * b), nr, true, m, st));
+  else RF_TRY(prod_c(op, false, W.Lq, W.vp, nr, true, c2(1.0 / (k * b), 0.0), false, m, st, fd));
   // zp = L^+ Sigma^T up
   RF_K(sigma_t(g, W.up, W.s, nr, st, make_feed(op, fd, C, m, W.z)));
   RF_TRY(prod_r(op, *op->lplus, W.s, W.z, nr, 1.0, false, m, st, fd));
@@ -1985,9 +2010,15 @@ int rfcmp_apply(rfcmp_op* op, int which, const rfcmp_c128* xin, rfcmp_c128* yout
     case RFCMP_APPLY_T:
     case RFCMP_APPLY_T_ADJ: {
       const bool adj = which == RFCMP_APPLY_T_ADJ;
-      RF_K(sigma_t(op->g, x, W.s, nr, st));
-      RF_TRY(prod_c(op, false, W.s, W.w, nr, adj, c2(1, 0), false, m, st));
-      RF_TRY(prod_c(op, true, x, W.u, nr, adj, c2(1, 0), false, m, st));
+      if (gemv_feedable(op, nr, m) && gemv_pairs(nr, m, W.gs)) {
+        RF_K(sigma_t(op->g, x, W.s, nr, st, make_feed(op, true, C, m, W.w, nullptr, 1)));
+        RF_K(gemv_split(x, W.u, N, nr, m, W.gs, st));
+        RF_TRY(prod_pair(op, W.u, W.w, 1.0, nr, adj, m, st));
+      } else {
+        RF_K(sigma_t(op->g, x, W.s, nr, st));
+        RF_TRY(prod_c(op, false, W.s, W.w, nr, adj, c2(1, 0), false, m, st));
+        RF_TRY(prod_c(op, true, x, W.u, nr, adj, c2(1, 0), false, m, st));
+      }
       // T x = i k T_A x - (i/k) Sigma V Sigma^T x ; T^H x = -i k conj(T_A) x + (i/k) Sigma conj(V) Sigma^T x
       EdgeCombo c;
       c.x = W.u;

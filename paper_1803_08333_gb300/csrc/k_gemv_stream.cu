@@ -104,6 +104,16 @@ struct Ring {
   }
 };
 
+// One product of a launch, and which of two a CTA works on: CTAs 0 .. split - 1 the first.
+struct GemvJob {
+  const void* M;
+  const float2 *xh, *xl;
+  double2* out;
+  double scale;
+  long long units;
+  int ld, n;
+};
+
 // ---------------------------------------------------------------- symmetric matrices
 // For a symmetric M (T_A, V and the factors all are) only the tiles that reach the diagonal or
 // lie above it are read: a tile of 8 rows I x one segment J contributes y_I += M_IJ x_J (row part,
@@ -228,9 +238,18 @@ __device__ __forceinline__ void sym_tile(const uint8_t* st, int qc, int row0, in
 
 template <int NR, bool REAL, bool CONJ, int NCTA>
 __global__ void __launch_bounds__(STHREADS, NCTA)
-gemv_sym_kernel(const void* __restrict__ Mv, int ld, int n, const float2* __restrict__ xh,
-                double2* __restrict__ out, double scale, long long units, int* __restrict__ err) {
+gemv_sym_kernel(const __grid_constant__ GemvJob J0, const __grid_constant__ GemvJob J1, int split,
+                int* __restrict__ err) {
   RF_COUNT_LAUNCH();
+  const bool other = (int)blockIdx.x >= split;
+  const GemvJob& J = other ? J1 : J0;
+  const int bid = other ? blockIdx.x - split : blockIdx.x, ctas = other ? gridDim.x - split : split;
+  const void* __restrict__ Mv = J.M;
+  const float2* __restrict__ xh = J.xh;
+  double2* __restrict__ out = J.out;
+  const double scale = J.scale;
+  const long long units = J.units;
+  const int ld = J.ld, n = J.n;
   constexpr int NST = SymStage<NR, REAL, NCTA>::NST;
   constexpr int STG = SymStage<NR, REAL, NCTA>::BYTES;
   constexpr int XB = SymStage<NR, REAL, NCTA>::XB;
@@ -247,7 +266,7 @@ gemv_sym_kernel(const void* __restrict__ Mv, int ld, int n, const float2* __rest
   static_assert(V == 16 || V == 32, "reduce-scatter of 16 or 32 values");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const SymGeom G = sym_geom(n, ld, SEG);
-  const long long u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
+  const long long u0 = units * bid / ctas, u1 = units * (bid + 1) / ctas;
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
       mbar_init(&full[s], 1);
@@ -448,17 +467,26 @@ __device__ __forceinline__ void ff_acc(f32x2& hi, f32x2& lo, f32x2 a, f32x2 bh, 
 }
 template <bool CONJ>
 __global__ void __launch_bounds__(STHREADS, FF_NCTA)
-gemv_stream_ff_kernel(const float2* __restrict__ M, int ld, int n, const float2* __restrict__ xh,
-                      const float2* __restrict__ xl, double2* __restrict__ out, double scale, long long units,
-                      int upr, int* __restrict__ err) {
+gemv_stream_ff_kernel(const __grid_constant__ GemvJob J0, const __grid_constant__ GemvJob J1, int split,
+                      int* __restrict__ err) {
   RF_COUNT_LAUNCH();
+  const bool other = (int)blockIdx.x >= split;
+  const GemvJob& J = other ? J1 : J0;
+  const int bid = other ? blockIdx.x - split : blockIdx.x, ctas = other ? gridDim.x - split : split;
+  const float2* __restrict__ M = static_cast<const float2*>(J.M);
+  const float2 *__restrict__ xh = J.xh, *__restrict__ xl = J.xl;
+  double2* __restrict__ out = J.out;
+  const double scale = J.scale;
+  const long long units = J.units;
+  const int ld = J.ld, n = J.n;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + FF_NST * FF_STAGE);
   uint64_t* empty = full + FF_NST;
   constexpr int SEG = FF_ROW / 8;  // complex entries per row segment
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
+  const int upr = (ld + SEG - 1) / SEG;
+  const long long u0 = units * bid / ctas, u1 = units * (bid + 1) / ctas;
   const int cnt = (int)(u1 - u0), rb0 = (int)(u0 / upr), cc0 = (int)(u0 % upr);
   if (threadIdx.x == 0) {
     for (int s = 0; s < FF_NST; ++s) {
@@ -860,8 +888,16 @@ gemv_sym_ff_kernel(const char* __restrict__ M, const char* __restrict__ Mlo, int
 // the register file): twice the warps to hide the consumers' latency (complex T_A product at
 // N = 30720: 0.659 ms with one CTA of four stages, 0.585 ms with two CTAs of two stages,
 // 0.557 ms with two CTAs of three stages: the measured copy bandwidth).
+// CTAs of the first of two jobs (b may be empty): in proportion to their units, at least one each
+int gemv_split_ctas(const GemvJob& a, const GemvJob& b, int grid) {
+  if (b.units == 0) return grid;
+  long long g = (grid * a.units + (a.units + b.units) / 2) / (a.units + b.units);
+  g = std::max<long long>(std::max<long long>(1, grid - b.units), std::min<long long>(g, std::min<long long>(grid - 1, a.units)));
+  return (int)g;
+}
+
 template <int NR, bool REAL, bool CONJ>
-cudaError_t launch_sym(const void* M, int ld, int n, GemvScratch& w, cudaStream_t s) {
+cudaError_t launch_sym(GemvJob a, GemvJob b, GemvScratch& w, cudaStream_t s) {
   constexpr int SEG = SBYTES_ROW / (REAL ? 4 : 8);
   constexpr int NCTA = REAL && NR == 2 ? 1 : 2;
   constexpr int SMEM = SymStage<NR, REAL, NCTA>::SMEM;
@@ -877,15 +913,18 @@ cudaError_t launch_sym(const void* M, int ld, int n, GemvScratch& w, cudaStream_
   });
   if (attr != cudaSuccess) return attr;
   if (!w.err) return cudaErrorInvalidValue;
-  const SymGeom G = sym_geom(n, ld, SEG);
-  const long long units = G.off(G.S);
-  const int grid = (int)std::max(1LL, std::min<long long>(units, (long long)NCTA * sms));
-  k<<<grid, STHREADS, SMEM, s>>>(M, ld, n, w.xh, w.out, w.scale, units, w.err);
+  for (GemvJob* q : {&a, &b}) {
+    if (q->n <= 0) continue;
+    const SymGeom G = sym_geom(q->n, q->ld, SEG);
+    q->units = G.off(G.S);
+  }
+  const int grid = (int)std::max(1LL, std::min<long long>(a.units + b.units, (long long)NCTA * sms));
+  k<<<grid, STHREADS, SMEM, s>>>(a, b, gemv_split_ctas(a, b, grid), w.err);
   return cudaGetLastError();
 }
 
 template <bool CONJ>
-cudaError_t launch_stream_ff(const float2* M, int ld, int n, GemvScratch& w, cudaStream_t s) {
+cudaError_t launch_stream_ff(GemvJob a, GemvJob b, GemvScratch& w, cudaStream_t s) {
   constexpr int SEG = FF_ROW / 8;
   auto k = gemv_stream_ff_kernel<CONJ>;
   static std::once_flag once;
@@ -899,11 +938,17 @@ cudaError_t launch_stream_ff(const float2* M, int ld, int n, GemvScratch& w, cud
   });
   if (attr != cudaSuccess) return attr;
   if (!w.err || !w.xl) return cudaErrorInvalidValue;
-  const int upr = (ld + SEG - 1) / SEG;
-  const long long units = (long long)((n + SROWS - 1) / SROWS) * upr;
-  const int grid = (int)std::max(1LL, std::min<long long>(units, (long long)FF_NCTA * sms));
-  k<<<grid, STHREADS, FF_NST * FF_STAGE + 256, s>>>(M, ld, n, w.xh, w.xl, w.out, w.scale, units, upr, w.err);
+  for (GemvJob* q : {&a, &b}) {
+    if (q->n <= 0) continue;
+    q->units = (long long)((q->n + SROWS - 1) / SROWS) * ((q->ld + SEG - 1) / SEG);
+  }
+  const int grid = (int)std::max(1LL, std::min<long long>(a.units + b.units, (long long)FF_NCTA * sms));
+  k<<<grid, STHREADS, FF_NST * FF_STAGE + 256, s>>>(a, b, gemv_split_ctas(a, b, grid), w.err);
   return cudaGetLastError();
+}
+
+GemvJob gemv_job(const void* M, int ld, int n, const GemvScratch& w) {
+  return GemvJob{M, w.xh, w.xl, w.out, w.scale, 0, ld, n};
 }
 
 template <bool REAL, bool CONJ>
@@ -934,22 +979,39 @@ cudaError_t launch_sym_ff(const void* M, const void* Mlo, int ld, int n, int nr,
 template <int NR>
 cudaError_t gemv_stream_c64(const float2* M, int ld, int n, bool conj, GemvScratch& w, cudaStream_t s) {
   if (!w.symmetric) return cudaErrorInvalidValue;
-  return conj ? launch_sym<NR, false, true>(M, ld, n, w, s) : launch_sym<NR, false, false>(M, ld, n, w, s);
+  const GemvJob a = gemv_job(M, ld, n, w);
+  return conj ? launch_sym<NR, false, true>(a, GemvJob{}, w, s) : launch_sym<NR, false, false>(a, GemvJob{}, w, s);
 }
 template <int NR>
 cudaError_t gemv_stream_r32(const float* M, int ld, int n, GemvScratch& w, cudaStream_t s) {
   if (!w.symmetric) return cudaErrorInvalidValue;
-  return launch_sym<NR, true, false>(M, ld, n, w, s);
+  return launch_sym<NR, true, false>(gemv_job(M, ld, n, w), GemvJob{}, w, s);
 }
 cudaError_t gemv_stream_c64_ff(const float2* M, int ld, int n, int nr, bool conj, GemvScratch& w, cudaStream_t s) {
   // One complex column takes the full pass: 1.46 ms against 1.8 here at N = 30720, where neither waits for HBM
   // (7.55 GB in 1.11 ms) and the pass over whole rows keeps no column sums.
-  if (nr == 1) return conj ? launch_stream_ff<true>(M, ld, n, w, s) : launch_stream_ff<false>(M, ld, n, w, s);
+  const GemvJob a = gemv_job(M, ld, n, w);
+  if (nr == 1) return conj ? launch_stream_ff<true>(a, GemvJob{}, w, s) : launch_stream_ff<false>(a, GemvJob{}, w, s);
   return conj ? launch_sym_ff<false, true>(M, nullptr, ld, n, nr, w, s)
               : launch_sym_ff<false, false>(M, nullptr, ld, n, nr, w, s);
 }
 cudaError_t gemv_stream_r32_ff(const float* hi, const float* lo, int ld, int n, int nr, GemvScratch& w, cudaStream_t s) {
   return launch_sym_ff<true, false>(hi, lo, ld, n, nr, w, s);
+}
+cudaError_t gemv_stream_pair(const GemvPart& a, const GemvPart& b, int nr, bool conj, GemvMode mode, GemvScratch& w,
+                             cudaStream_t s) {
+  if (!w.symmetric) return cudaErrorInvalidValue;
+  GemvJob J[2];
+  for (int i = 0; i < 2; ++i) {
+    const GemvPart& p = i ? b : a;
+    J[i] = GemvJob{p.M, p.xh, p.xl, p.out, p.scale, 0, padded_ld(p.n), p.n};
+  }
+  if (mode == GEMV_FF) {
+    if (nr != 1) return cudaErrorInvalidValue;
+    return conj ? launch_stream_ff<true>(J[0], J[1], w, s) : launch_stream_ff<false>(J[0], J[1], w, s);
+  }
+  if (nr == 1) return conj ? launch_sym<1, false, true>(J[0], J[1], w, s) : launch_sym<1, false, false>(J[0], J[1], w, s);
+  return conj ? launch_sym<2, false, true>(J[0], J[1], w, s) : launch_sym<2, false, false>(J[0], J[1], w, s);
 }
 template cudaError_t gemv_stream_c64<1>(const float2*, int, int, bool, GemvScratch&, cudaStream_t);
 template cudaError_t gemv_stream_c64<2>(const float2*, int, int, bool, GemvScratch&, cudaStream_t);

@@ -459,6 +459,30 @@ cudaError_t gemv_c64(const float2* M, int n, const double2* x, double2* y, int n
   return err;
 }
 
+// A launch and its empty SMs cost a small body as much as a product: T of one column, 480 functions and 320 cells, 29 us
+// with a launch for each product, 24 in one; a solve of 1920 functions and 1280 cells 4.55 and 4.00 ms.  Large products
+// neither gain nor lose (30720 functions: 6.54 and 6.56 ms for A).
+bool gemv_pairs(int nr, GemvMode mode, const GemvScratch& w) {
+  return (mode == GEMV_F32 ? nr == 1 || nr == 2 : nr == 1) && w.chunk == 0 && w.ctas_per_sm == 0 && w.err && w.symmetric;
+}
+cudaError_t gemv_c64_pair(const GemvPart& a, const GemvPart& b, int nr, bool conj, GemvMode mode, GemvScratch& w,
+                          cudaStream_t s) {
+  if (!gemv_pairs(nr, mode, w)) return cudaErrorInvalidValue;
+  double bytes = 0.0, flops = 0.0;
+  for (const GemvPart* p : {&a, &b}) {
+    const double n = p->n;
+    bytes += (mode == GEMV_F32 ? 4.0 * n * (n + 1.0) : 8.0 * n * n) + 32.0 * n * nr;
+    flops += 8.0 * n * n * nr;
+  }
+  ProfScope prof(mode == GEMV_FF ? "gemv_c64_ff" : "gemv_c64_f32", bytes, flops, s, 2);
+  return gemv_stream_pair(a, b, nr, conj, mode, w, s);
+}
+cudaError_t gemv_split(const double2* x, double2* y, int n, int nr, GemvMode mode, GemvScratch& w, cudaStream_t s) {
+  const int ld = padded_ld(n);
+  if (n > w.cap_n || ld > w.cap_ld || nr > w.cap_cols) return cudaErrorInvalidValue;
+  return gemv_prep(x, y, n, ld, nr, mode == GEMV_FF, false, 1.0, w, s);
+}
+
 // The same complex GEMV without profiling events and without the cached grid map: it
 // performs no allocation of any kind (device, driver or host heap).
 cudaError_t gemv_c64_plain(const float2* M, int n, const double2* x, double2* y, int nrhs, bool conjugate,

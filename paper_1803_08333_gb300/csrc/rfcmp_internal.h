@@ -73,13 +73,14 @@ int set_error(int code, const std::string& msg);
 // RAII bracket of one launch by CUDA events on its stream (no-op when disabled).
 class ProfScope {
  public:
-  ProfScope(const char* family, double bytes, double flops, cudaStream_t s);
+  // products: how many of the family's products the launch does (it counts as that many launches)
+  ProfScope(const char* family, double bytes, double flops, cudaStream_t s, int products = 1);
   ~ProfScope();
   ProfScope(const ProfScope&) = delete;
   ProfScope& operator=(const ProfScope&) = delete;
 
  private:
-  int slot_ = -1;
+  int slot_ = -1, products_ = 1;
   cudaStream_t s_ = nullptr;
   cudaEvent_t a_ = nullptr, b_ = nullptr;  // this launch's own start / end events
   uint64_t gen_ = 0;                        // profiling generation the slot belongs to
@@ -294,6 +295,17 @@ template <int NR>
 cudaError_t gemv_stream_c64(const float2* M, int ld, int n, bool conj, GemvScratch& w, cudaStream_t s);
 template <int NR>
 cudaError_t gemv_stream_r32(const float* M, int ld, int n, GemvScratch& w, cudaStream_t s);
+// Two such products in one launch: one column in float-float, or one or two in FP32 (mode), each matrix with its own
+// prepared x, output and scale.
+struct GemvPart {
+  const float2* M = nullptr;
+  int n = 0;
+  const float2 *xh = nullptr, *xl = nullptr;
+  double2* out = nullptr;
+  double scale = 1.0;
+};
+cudaError_t gemv_stream_pair(const GemvPart& a, const GemvPart& b, int nr, bool conj, GemvMode mode, GemvScratch& w,
+                             cudaStream_t s);
 // Float-float streaming GEMV of nr columns of a symmetric complex64 M, or FP32 hi + lo one (x split in
 // w.xh + w.xl).
 cudaError_t gemv_stream_c64_ff(const float2* M, int ld, int n, int nr, bool conj, GemvScratch& w, cudaStream_t s);
@@ -324,6 +336,12 @@ void dev_pool_trim();
 cudaError_t gemv_c64(const float2* M, int n, const double2* x, double2* y, int nrhs, bool conjugate,
                      double2 scale, bool accumulate, GemvMode mode, GemvScratch& w, cudaStream_t s,
                      bool fed = false);
+// whether gemv_c64_pair takes nr columns in this mode with this scratch (its own split of x for either matrix)
+bool gemv_pairs(int nr, GemvMode mode, const GemvScratch& w);
+cudaError_t gemv_c64_pair(const GemvPart& a, const GemvPart& b, int nr, bool conj, GemvMode mode, GemvScratch& w,
+                          cudaStream_t s);
+// the split of x for a following product (w.xh, w.xl), y zeroed
+cudaError_t gemv_split(const double2* x, double2* y, int n, int nr, GemvMode mode, GemvScratch& w, cudaStream_t s);
 // y = op(M) x through the same kernels with no allocation of any kind (no profiling events,
 // no cached launch-grid table).
 cudaError_t gemv_c64_plain(const float2* M, int n, const double2* x, double2* y, int nrhs, bool conjugate,
