@@ -428,7 +428,8 @@ __device__ Pot triangle_potentials(const double r[3], const CellFrame& f) {
       den = R02;
     }
     double F = 0.0;
-    if (!in || R02 > 1e-30 * f.len[i] * f.len[i]) F = log(num / den);
+    // on the edge's line F's factors p0 and R0^2 vanish, and at a corner num / den is not finite
+    if (R02 > 1e-30 * f.len[i] * f.len[i]) F = log(num / den);
     out.S = fma(p0, F, out.S);
     const double c = 0.5 * fma(R02, F, fma(lp, Rp, -lm * Rm));
 #pragma unroll
