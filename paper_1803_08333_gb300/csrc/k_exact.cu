@@ -82,6 +82,9 @@ struct ExactMaps {
 constexpr int XTHREADS = 320;  // producer warp, MMA warp, 8 epilogue warps
 static_assert(XBN == 32, "two epilogue warps of 16 columns per tensor-memory quadrant");
 
+constexpr int NOT_FINITE = INT_MIN;  // exponent of a column with an infinity or a NaN: its products are NaN
+__device__ __forceinline__ double quiet_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
+
 __global__ void __launch_bounds__(XTHREADS, 1)
 exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, const int* __restrict__ ea,
                   const int* __restrict__ eb, double* __restrict__ D, longlong2* __restrict__ DI, long long ldd,
@@ -230,8 +233,8 @@ exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, c
       for (int j = 0; j < 16; ++j) {
         const int col = n0 + h + j;
         if (col < N) {
-          const int e = er + eb[col];
-          dst[col] = ldexp((double)H[j], e - 32) + ldexp((double)G[j], e - 56);
+          const int x = eb[col], e = er + (x == NOT_FINITE ? 0 : x);
+          dst[col] = x == NOT_FINITE ? quiet_nan() : ldexp((double)H[j], e - 32) + ldexp((double)G[j], e - 56);
         }
       }
     }
@@ -247,7 +250,6 @@ exact_gemm_kernel(const __grid_constant__ ExactMaps maps, int M, int N, int K, c
 // operations, 128 added to each so that the bytes are the digits plus 128 (GB300's FP64 pipe runs at
 // 1/64 of the integer rate; in FP64 the digits of 16 columns of 7680 took 48 us, and now 7).
 constexpr unsigned long long DIGIT_BIAS = 0x808080808080ull;
-constexpr int NOT_FINITE = INT_MIN;  // exponent of a column with an infinity or a NaN: its products are NaN
 
 // m 2^-s rounded to an integer
 __device__ __forceinline__ unsigned long long shift_round(unsigned long long m, int s) {
@@ -395,7 +397,7 @@ combine_int_kernel(const longlong2* __restrict__ D, const int* __restrict__ ea, 
   auto value = [&](int row, int col) {
     const longlong2 d = D[(size_t)row * (2 * nr) + col];
     const int x = eb[col];
-    if (x == NOT_FINITE) return __longlong_as_double(0x7ff8000000000000ll);
+    if (x == NOT_FINITE) return quiet_nan();
     const int e = ea[row] + x;
     return ldexp((double)d.x, e - 32) + ldexp((double)d.y, e - 56);
   };
