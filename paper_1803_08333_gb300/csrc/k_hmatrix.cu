@@ -708,8 +708,10 @@ struct HmPart {
 // Frees the temporaries of one build on every path out of it.
 struct HmTemps {
   std::vector<void*> p;
-  ~HmTemps() {
+  ~HmTemps() { clear(); }
+  void clear() {
     for (void* q : p) dev_free(q);
+    p.clear();
   }
   template <class T>
   cudaError_t alloc(T** q, size_t bytes) {
@@ -859,7 +861,8 @@ int start_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, uint64_t 
 }
 
 // Waits for the cross approximations and packs the final blocks: the admissible ones whose crosses met the
-// stopping rule in low rank, the rest dense.
+// stopping rule in low rank, the rest dense.  The slots and lists of the approximations end here (freed after the
+// packing on its stream), so that one matrix's are not held beside the other's.
 int finish_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, PartBuild& b, HmPart& out,
                 std::vector<void*>& owned) {
   const int cap = o.max_rank;
@@ -913,6 +916,7 @@ int finish_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, PartBuil
     hm_pack_kernel<<<(unsigned)fin.size(), HM_THREADS>>>(A, ld, out.perm, out.blocks, fslot_d, cap, b.slots, out.data);
     HM_CUDA(cudaGetLastError());
   }
+  b.tmp.clear();
   const std::vector<int2> items = cross_items(fin);
   out.nitems = (int)items.size();
   out.ntiles = (int)lists.tiles.size();
@@ -1049,8 +1053,8 @@ int rfcmp_hm_create(rfcmp_op* op, const rfcmp_hm_opts* opts_in, rfcmp_hm** out) 
     const float2* mats[2] = {v.TA, v.V};
     const int lds[2] = {v.ldN, v.ldC}, ns[2] = {v.n, v.nc};
     PartBuild part[2];
-    // the host partitions V beside T_A (a thread of its own, or after it where none can be had) and, where
-    // no budget orders the two, while T_A's crosses are found
+    // the host partitions V beside T_A (a thread of its own, or after it where none can be had); the builds
+    // follow one another, so that the peak is one matrix's slots
     auto split_v = [&] { partition(ccen.data(), clo.data(), chi.data(), v.nc, o.leaf, o.eta, part[1].perm, part[1].blocks); };
     std::future<void> other;
     try {
@@ -1058,7 +1062,6 @@ int rfcmp_hm_create(rfcmp_op* op, const rfcmp_hm_opts* opts_in, rfcmp_hm** out) 
     } catch (const std::system_error&) {
     }
     partition(ecen.data(), elo.data(), ehi.data(), v.n, o.leaf, o.eta, part[0].perm, part[0].blocks);
-    const bool together = v.budget == 0;
     for (int w = 0; w < 2 && rc == RFCMP_OK; ++w) {
       uint64_t left = UINT64_MAX;
       if (v.budget) {
@@ -1070,11 +1073,8 @@ int rfcmp_hm_create(rfcmp_op* op, const rfcmp_hm_opts* opts_in, rfcmp_hm** out) 
         else split_v();
       }
       rc = start_part(mats[w], lds[w], ns[w], o, left, part[w], hm->part[w], hm->owned);
-      if (rc != RFCMP_OK || (together && w == 0)) continue;
-      for (int z = together ? 0 : w; z <= w && rc == RFCMP_OK; ++z) {
-        rc = finish_part(mats[z], lds[z], ns[z], o, part[z], hm->part[z], hm->owned);
-        hm->bytes += hm->part[z].bytes;
-      }
+      if (rc == RFCMP_OK) rc = finish_part(mats[w], lds[w], ns[w], o, part[w], hm->part[w], hm->owned);
+      hm->bytes += hm->part[w].bytes;
     }
   } catch (const std::bad_alloc&) {
     return set_error(RFCMP_ERR_CUDA, "out of host memory");
