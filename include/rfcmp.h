@@ -506,8 +506,8 @@ int rfcmp_hm_partition(const double* centres, const double* sup_lo, const double
 /* Compresses op's T_A and V (opts NULL for the defaults).  Runs on the context device's legacy
  * default stream and returns when the compressed form is ready.  Its bytes count against the
  * context's budget; destroy it before the context.
- * Errors: RFCMP_ERR_INVALID_ARG, RFCMP_ERR_OUT_OF_BUDGET (the build's peak: the crosses' slots
- * and, at worst, every block dense), RFCMP_ERR_CUDA. */
+ * Errors: RFCMP_ERR_INVALID_ARG, RFCMP_ERR_OUT_OF_BUDGET (the build's peak, T_A's and then V's: at
+ * worst every block dense, and the crosses' slots or the product's lists), RFCMP_ERR_CUDA. */
 int rfcmp_hm_create(rfcmp_op* op, const rfcmp_hm_opts* opts, rfcmp_hm** out);
 
 /* y = H x for nrhs columns, H the compressed T_A or V (which), FP32 factors with FP64

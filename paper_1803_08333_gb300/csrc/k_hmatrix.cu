@@ -784,10 +784,11 @@ std::vector<int2> cross_items(const std::vector<HmBlockDev>& blk) {
 
 template <class T>
 cudaError_t keep(T** d, const std::vector<T>& h, std::vector<void*>& owned) {
-  cudaError_t e = dev_malloc(d, std::max<size_t>(h.size() * sizeof(T), 8));
+  if (h.empty()) return cudaSuccess;
+  cudaError_t e = dev_malloc(d, h.size() * sizeof(T));
   if (e != cudaSuccess) return e;
   owned.push_back(*d);
-  return h.empty() ? cudaSuccess : cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
+  return cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
 }
 
 // One matrix on its way to the compressed form: the partition (host), the cross approximations (queued
@@ -799,6 +800,7 @@ struct PartBuild {
   std::vector<long long> slot;
   int32_t *rank_d = nullptr, *status_d = nullptr;
   float2* slots = nullptr;
+  CoverLists lists;
   HmTemps tmp;
 };
 
@@ -811,19 +813,30 @@ int start_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, uint64_t 
   const int cap = o.max_rank;
   std::vector<int32_t> order;  // candidates, the large ones (a CTA each) before the small ones (a warp each)
   long long slot_elems = 0, worst = 0;
+  uint64_t item_bytes = 0;
   for (const HmBlockHost& h : b.blocks) {
     const long long m = h.r1 - h.r0, nn = h.c1 - h.c0;
-    worst += m * nn;  // the peak holds the slots and, at worst, every block dense
+    worst += m * nn;  // at worst every block is stored dense
     if (h.admissible) {
       b.cand.push_back({h.r0, h.r1, h.c0, h.c1, 0, 0, 0});
       b.slot.push_back(slot_elems);
       slot_elems += (long long)cap * (m + nn);
+      // a low-rank block keeps fewer crosses than make its own entries
+      const long long most = std::min<long long>(cap, m * nn / (m + nn));
+      item_bytes += 2 * sizeof(int2) * (uint64_t)((most + HM_CROSS - 1) / HM_CROSS);
     }
   }
-  const uint64_t peak = 8ull * (uint64_t)(slot_elems + worst) + 64ull * b.blocks.size() + 4ull * n;
-  if (budget_left != UINT64_MAX && peak > budget_left)
-    return set_error(RFCMP_ERR_OUT_OF_BUDGET, "compression needs up to " + std::to_string(peak) + " bytes, budget has " +
-                                                  std::to_string(budget_left));
+  if (budget_left != UINT64_MAX) {
+    // the blocks and, beside them, first the slots and lists of the approximations, then the lists of the product
+    b.lists = cover_lists(b.blocks, n);
+    const uint64_t nb = b.blocks.size(), nc = b.cand.size();
+    const uint64_t temps = 8ull * (uint64_t)slot_elems + nc * (sizeof(HmBlockDev) + 20) + 8 * nb;
+    const uint64_t keeps = item_bytes + sizeof(HmTile) * b.lists.tiles.size() + 4ull * b.lists.cover.size();
+    const uint64_t peak = 8ull * (uint64_t)worst + sizeof(HmBlockDev) * nb + 4ull * n + std::max(temps, keeps);
+    if (peak > budget_left)
+      return set_error(RFCMP_ERR_OUT_OF_BUDGET, "compression needs up to " + std::to_string(peak) +
+                                                    " bytes, budget has " + std::to_string(budget_left));
+  }
   HM_CUDA(dev_malloc(&out.perm, std::max<size_t>(4 * (size_t)n, 4)));
   owned.push_back(out.perm);
   if (n > 0) HM_CUDA(cudaMemcpy(out.perm, b.perm.data(), 4 * (size_t)n, cudaMemcpyHostToDevice));
@@ -861,12 +874,13 @@ int start_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, uint64_t 
 }
 
 // Waits for the cross approximations and packs the final blocks: the admissible ones whose crosses met the
-// stopping rule in low rank, the rest dense.  The slots and lists of the approximations end here (freed after the
-// packing on its stream), so that one matrix's are not held beside the other's.
+// stopping rule in low rank, the rest dense.  The slots and lists of the approximations end here, so that
+// one matrix's are not held beside the other's, nor beside the product's lists.
 int finish_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, PartBuild& b, HmPart& out,
                 std::vector<void*>& owned) {
   const int cap = o.max_rank;
-  const CoverLists lists = cover_lists(b.blocks, n);  // while the crosses are found
+  if (b.lists.tiles.empty()) b.lists = cover_lists(b.blocks, n);  // while the crosses are found
+  const CoverLists& lists = b.lists;
   std::vector<int32_t> rank(b.cand.size(), 0), status(b.cand.size(), 1);
   if (!b.cand.empty()) {
     HM_CUDA(cudaMemcpy(rank.data(), b.rank_d, 4 * b.cand.size(), cudaMemcpyDeviceToHost));
@@ -916,14 +930,14 @@ int finish_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, PartBuil
     hm_pack_kernel<<<(unsigned)fin.size(), HM_THREADS>>>(A, ld, out.perm, out.blocks, fslot_d, cap, b.slots, out.data);
     HM_CUDA(cudaGetLastError());
   }
-  b.tmp.clear();
   const std::vector<int2> items = cross_items(fin);
+  b.tmp.clear();
+  HM_CUDA(cudaStreamSynchronize(0));  // packed, and the pool has the temporaries back
   out.nitems = (int)items.size();
   out.ntiles = (int)lists.tiles.size();
   HM_CUDA(keep(&out.items, items, owned));
   HM_CUDA(keep(&out.tiles, lists.tiles, owned));
   HM_CUDA(keep(&out.cover, lists.cover, owned));
-  HM_CUDA(cudaStreamSynchronize(0));
   out.bytes = 8ull * (uint64_t)off + sizeof(HmBlockDev) * fin.size() + 4ull * n + sizeof(int2) * items.size() +
               sizeof(HmTile) * lists.tiles.size() + 4ull * lists.cover.size();
   return RFCMP_OK;

@@ -28,8 +28,8 @@ def _peak(op, **opts):
     return s["used_high"] - before, s["used"] - before
 
 
-# slots of many crosses, and of one
-@pytest.mark.parametrize("level,leaf,max_rank", [(10, 32, 256), (8, 8, 64), (7, 16, 1)])
+# slots of many crosses; of one; no admissible block at all
+@pytest.mark.parametrize("level,leaf,max_rank", [(10, 32, 256), (8, 8, 64), (7, 16, 1), (4, 1000, 64), (9, 600, 64)])
 def test_peak_is_the_stated_one(level, leaf, max_rank):
     from paper_1803_08333_gb300 import build
 
