@@ -60,7 +60,14 @@ def op_footprint(nv: int, nc: int, nrhs: int, with_factors: bool, widest: int = 
         return b
 
     base = 0 if widest else 8 * cplx + (8 * real + 64 * nc * nc if with_factors else 0)
-    vectors = 16 * ne * max(nrhs, 4) * 24 if nrhs > widest else 0
+    vectors = 0
+    if nrhs > widest:
+        # 24 vectors a column of the workspace and the solve, the staging of a session, scalars and partial sums
+        vectors = (16 * 25 * ne + 1024) * max(nrhs, 4)
+        if nrhs >= 4:
+            # results of the tensor-core products: pairs of 64-bit integers up to 32 columns where FP64 values take
+            # half of that, and 161 tile slots of 128 rows (Re and Im, at most 64 columns) beside D
+            vectors += 8 * ne * max(0, 8 * min(nrhs, 32) - 4 * nrhs) + 4 * 161 * 256 * min(nrhs, 64)
     return base + extra(nrhs) - extra(widest) + vectors
 
 
