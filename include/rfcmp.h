@@ -427,6 +427,16 @@ int rfcmp_pool_reset_high(void);
 /* Hands the memory the pool holds but no buffer uses back to the driver (synchronises the device). */
 int rfcmp_pool_trim(void);
 
+/* x <- (I - J) M (I - J) + J, J = 1 1^T / n, M one multigrid V(1,1) cycle for the Laplacian of a connected graph:
+ * the approximation of (L + J)^{-1} that the refinement of (Sigma^T Sigma)^+ starts from (the paper
+ * has no counterpart: for checks of it).
+ *  ptr, col, val  L in CSR (host), symmetric with a positive diagonal; more than 64 rows (fewer: no level).
+ *  rows           0 applies the cycle to the columns of I - J; 1 to 4 builds it as a matrix, at most so many
+ *                 rows (1, 2 or 4) sharing a CTA; beyond 28160 rows on a coarse level as 0.
+ *  x              n x n float64 row-major, DEVICE memory of the current device.  Synchronises.
+ * Errors: RFCMP_ERR_INVALID_ARG (NULL, n not in [1, 65535], indices out of range, no level), RFCMP_ERR_CUDA. */
+int rfcmp_vcycle_start(const int32_t* ptr, const int32_t* col, const double* val, int64_t n, int32_t rows, double* x);
+
 /* How rfcmp_solve runs its loop (the paper has no counterpart; the arithmetic is the same
  * either way, so the results are identical).  Nonzero (the default, unless the environment
  * variable RFCMP_SOLVE_GRAPHS is "0" when the first solve starts): refinement sweeps and CG

@@ -40,7 +40,7 @@ EXPORTED_SYMBOLS = [
     "rfcmp_pool_stats", "rfcmp_pool_reset_high", "rfcmp_pool_trim", "rfcmp_batch_create", "rfcmp_batch_destroy",
     "rfcmp_batch_admit", "rfcmp_batch_step", "rfcmp_batch_take", "rfcmp_batch_counts",
     "rfcmp_hm_opts_default", "rfcmp_hm_partition", "rfcmp_hm_create", "rfcmp_hm_apply", "rfcmp_hm_info_get",
-    "rfcmp_hm_destroy",
+    "rfcmp_hm_destroy", "rfcmp_vcycle_start",
 ]
 HM = {"T_A": 0, "V": 1}
 
@@ -186,6 +186,7 @@ def lib():
         u64p = ctypes.POINTER(ctypes.c_uint64)
         L.rfcmp_pool_stats.argtypes = [u64p, u64p, u64p, u64p]
         i32p = ctypes.POINTER(ctypes.c_int32)
+        L.rfcmp_vcycle_start.argtypes = [vp, vp, vp, i64, i32, vp]
         L.rfcmp_batch_create.argtypes = [vp, i32, ctypes.POINTER(SolveOpts), ctypes.POINTER(vp)]
         L.rfcmp_batch_destroy.argtypes = [vp]
         L.rfcmp_batch_admit.argtypes = [vp, vp, i32, i32p, vp]

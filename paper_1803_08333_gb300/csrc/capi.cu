@@ -1362,6 +1362,17 @@ std::vector<uint4> laplacian_rows(const std::vector<int32_t>& ptr, const std::ve
   return out;
 }
 
+// Xd (padded rows) <- one V-cycle of H as a matrix where multigrid_inverse takes it (*symmetric), else the V-cycle on
+// the columns of I - J
+cudaError_t vcycle_start(const AmgHierarchy& H, const int32_t* dptr, const int32_t* dcol, const double* dval, int n,
+                         int rows, double* Xd, int* iters, bool* symmetric) {
+  *iters = 0;
+  *symmetric = false;
+  const cudaError_t err = multigrid_inverse(H, n, Xd, padded_ld(n), symmetric, 0, rows);
+  if (err != cudaSuccess || *symmetric) return err;
+  return dense_inverse_block_cg(dptr, dcol, dval, n, true, &H, NS_START_TOL, 0, nullptr, nullptr, iters, 0, Xd);
+}
+
 // dense inverse of a sparse SPD matrix (CSR on the host), FP32 hi + lo planes
 int build_factor(const std::vector<int32_t>& ptr, const std::vector<int32_t>& col, const std::vector<double>& val,
                  int n, bool project, bool multigrid, double tol, std::shared_ptr<DenseFactor>& out,
@@ -1415,10 +1426,9 @@ int build_factor(const std::vector<int32_t>& ptr, const std::vector<int32_t>& co
     for (int attempt = 0; attempt < 2 && err == cudaSuccess && !(res <= accept); ++attempt) {
       int it = 0;
       bool start = false;
-      if (attempt == 0) err = multigrid_inverse(H, n, Xd, padded_ld(n), &start, 0);
-      if (err == cudaSuccess && !start)
-        err = dense_inverse_block_cg(dptr, dcol, dval, n, project, &H, NS_START_TOL, attempt == 0 ? 0 : 20000, f->hi,
-                                     f->lo, &it, 0, Xd);
+      if (attempt == 0) err = vcycle_start(H, dptr, dcol, dval, n, 4, Xd, &it, &start);
+      else
+        err = dense_inverse_block_cg(dptr, dcol, dval, n, true, &H, NS_START_TOL, 20000, nullptr, nullptr, &it, 0, Xd);
       iters += it;
       int st = 0;
       if (err == cudaSuccess)
@@ -1543,6 +1553,41 @@ int rfcmp_pool_stats(uint64_t* used, uint64_t* used_high, uint64_t* reserved, ui
 int rfcmp_pool_trim(void) {
   dev_pool_trim();
   RF_CUDA(cudaGetLastError());
+  return RFCMP_OK;
+}
+
+int rfcmp_vcycle_start(const int32_t* ptr, const int32_t* col, const double* val, int64_t n, int32_t rows, double* x) {
+  if (!ptr || !col || !val || !x || n < 1 || n > 65535 || rows < 0 || rows > 4 || ptr[0] != 0)
+    return set_error(RFCMP_ERR_INVALID_ARG, "invalid argument");
+  for (int64_t i = 0; i < n; ++i)
+    if (ptr[i + 1] < ptr[i]) return set_error(RFCMP_ERR_INVALID_ARG, "row pointers decrease");
+  for (int32_t q = 0; q < ptr[n]; ++q)
+    if (col[q] < 0 || col[q] >= n) return set_error(RFCMP_ERR_INVALID_ARG, "column out of range");
+  const std::vector<int32_t> hp(ptr, ptr + n + 1), hc(col, col + ptr[n]);
+  const std::vector<double> hv(val, val + ptr[n]);
+  AmgHierarchy H;
+  std::string msg;
+  const int rc = build_amg(hp, hc, hv, (int)n, 64, H, msg);
+  if (rc != RFCMP_OK) return set_error(rc, msg);
+  if (H.levels.empty()) return set_error(RFCMP_ERR_INVALID_ARG, "no multigrid level");
+  std::vector<void*> tmp;
+  struct Free {
+    std::vector<void*>& p;
+    ~Free() {
+      for (void* q : p) dev_free(q);
+    }
+  } free_all{tmp};
+  int32_t *dptr = nullptr, *dcol = nullptr;
+  double *dval = nullptr, *Xd = nullptr;
+  RF_TRY(upload(&dptr, hp, tmp));
+  RF_TRY(upload(&dcol, hc, tmp));
+  RF_TRY(upload(&dval, hv, tmp));
+  RF_TRY(dalloc(&Xd, (size_t)n * padded_ld((int)n), tmp));
+  int it = 0;
+  bool symmetric = false;
+  RF_K(vcycle_start(H, dptr, dcol, dval, (int)n, rows, Xd, &it, &symmetric));
+  RF_K(copy_rows(x, Xd, sizeof(double) * padded_ld((int)n), sizeof(double) * (size_t)n, (int)n, 0));
+  RF_CUDA(cudaStreamSynchronize(0));
   return RFCMP_OK;
 }
 

@@ -715,9 +715,10 @@ cudaError_t newton_schulz_pseudo_inverse(const int32_t* ptr, const int32_t* col,
   return fail(cudaSuccess);
 }
 
-cudaError_t multigrid_inverse(const AmgHierarchy& H, int n, double* X, long long ld, bool* done, cudaStream_t s) {
+cudaError_t multigrid_inverse(const AmgHierarchy& H, int n, double* X, long long ld, bool* done, cudaStream_t s,
+                              int rows) {
   *done = false;
-  if (H.levels.empty()) return cudaSuccess;
+  if (H.levels.empty() || rows < 1) return cudaSuccess;
   for (const AmgLevelHost& h : H.levels)
     if (sizeof(double) * (size_t)h.nc > (size_t)LIFT_SMEM) return cudaSuccess;
   *done = true;
@@ -777,9 +778,9 @@ cudaError_t multigrid_inverse(const AmgHierarchy& H, int n, double* X, long long
     const double* sh = l == 0 ? shift : nullptr;
     // four rows share the entries of S (and write whole sectors of the mirrored rows) where they fit
     const size_t row = sizeof(double) * (size_t)h.nc;
-    err = 4 * row <= (size_t)LIFT_SMEM   ? lift<4>(L, Mc, ldc, sh, M, ldm, s)
-          : 2 * row <= (size_t)LIFT_SMEM ? lift<2>(L, Mc, ldc, sh, M, ldm, s)
-                                         : lift<1>(L, Mc, ldc, sh, M, ldm, s);
+    err = rows >= 4 && 4 * row <= (size_t)LIFT_SMEM   ? lift<4>(L, Mc, ldc, sh, M, ldm, s)
+          : rows >= 2 && 2 * row <= (size_t)LIFT_SMEM ? lift<2>(L, Mc, ldc, sh, M, ldm, s)
+                                                      : lift<1>(L, Mc, ldc, sh, M, ldm, s);
     if (err != cudaSuccess) return fail(err);
     Mc = M;
     ldc = ldm;

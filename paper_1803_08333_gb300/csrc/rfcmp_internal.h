@@ -488,8 +488,9 @@ cudaError_t dense_inverse_block_cg(const int32_t* ptr, const int32_t* col, const
                                    int* iters, cudaStream_t s, double* Xd = nullptr);
 // X (n rows, stride ld) <- (I - J) M (I - J) + J, J = 1 1^T / n, M one V(1,1) cycle of H: an approximation of
 // (L + J)^{-1}, exactly symmetric (k_factor.cu).  *done = false, nothing queued, where the hierarchy has no
-// levels or a coarse row does not fit in shared memory.
-cudaError_t multigrid_inverse(const AmgHierarchy& H, int n, double* X, long long ld, bool* done, cudaStream_t s);
+// levels, a coarse row does not fit in shared memory or rows is 0.  rows: at most so many rows in a CTA's group.
+cudaError_t multigrid_inverse(const AmgHierarchy& H, int n, double* X, long long ld, bool* done, cudaStream_t s,
+                              int rows = 4);
 // hi + lo <- its symmetric part, in place (k_factor.cu)
 cudaError_t symmetrize_planes(float* hi, float* lo, int n, int ld, cudaStream_t s);
 // Newton-Schulz refinement of X ~ M^{-1} (k_factor.cu) for M = L + 1 1^T / n (project: writes
