@@ -102,10 +102,11 @@ __device__ __forceinline__ void seq_tile(int i, int tm, int tn, int upper, int& 
 
 // Work of CTA b of G: body(tile, q0, q1), the K blocks q0 .. q1 - 1 (of total) of an output tile, until it
 // returns false.  Whole tiles b, b + G, b + 2G, ..., or (split) an equal share of the K blocks of all tiles
-// in their order, at most one tile's end and another's start not its own.
-template <class F>
-__device__ __forceinline__ void gemm_pieces(int tiles, int total, int split, F&& body) {
-  if (split) {
+// in their order, at most one tile's end and another's start not its own.  Compiled apart: with the choice made in the
+// kernel the whole-tile products took 0.5 to 1 % longer.
+template <bool SPLIT, class F>
+__device__ __forceinline__ void gemm_pieces(int tiles, int total, F&& body) {
+  if constexpr (SPLIT) {
     const uint32_t T = (uint32_t)tiles * total, G = gridDim.x;
     uint32_t u = blockIdx.x * T / G;
     const uint32_t end = (blockIdx.x + 1) * T / G;
@@ -127,10 +128,10 @@ __device__ __forceinline__ void gemm_pieces(int tiles, int total, int split, F&&
 // tensor-memory buffer t % 2 while the epilogue warps drain buffer (t - 1) % 2, so a tile's
 // epilogue overlaps the next tile's main loop.  The epilogue goes through a shared-memory
 // transpose so that each warp store writes 128 contiguous bytes of one row of D.
-template <int BN>
+template <int BN, bool SPLIT>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask, int M, int N, int K,
-                   float* __restrict__ D, long long ldd, int accumulate, int* __restrict__ err, int upper, int split) {
+                   float* __restrict__ D, long long ldd, int accumulate, int* __restrict__ err, int upper) {
   RF_COUNT_LAUNCH();
   using C = TileCfg<BN>;
   constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, TILE_B = C::TILE_B;
@@ -178,7 +179,7 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
     if (lane == 0) {
       // producer: TMA loads into the stage ring, tile after tile
       long long it = 0;
-      gemm_pieces(tiles, total, split, [&](int lin, int q0, int q1) {
+      gemm_pieces<SPLIT>(tiles, total, [&](int lin, int q0, int q1) {
         int tile_m, tile_n;
         seq_tile(lin, tm, tn, upper, tile_m, tile_n);
         const int m0 = tile_m * BM, n0 = tile_n * BN;
@@ -209,7 +210,7 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
       const uint32_t id_pos = idesc_bf16(BM, BN, false), id_neg = idesc_bf16(BM, BN, true);
       long long it = 0;
       int t = 0;  // tiles of this CTA so far
-      gemm_pieces(tiles, total, split, [&](int, int q0, int q1) {
+      gemm_pieces<SPLIT>(tiles, total, [&](int, int q0, int q1) {
         const int b = t & 1, use = t >> 1;
         if (use > 0 && !mbar_wait(&acc_empty[b], (uint32_t)((use - 1) & 1))) {
           atomicExch(err, 5);
@@ -253,7 +254,7 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
     const int quarter = warp & 3;
     float* tb = epi + (warp - 2) * 32 * 33;
     int t = 0;
-    gemm_pieces(tiles, total, split, [&](int lin, int, int) {
+    gemm_pieces<SPLIT>(tiles, total, [&](int lin, int, int) {
       int tile_m, tile_n;
       seq_tile(lin, tm, tn, upper, tile_m, tile_n);
       const int b = t & 1, use = t >> 1;
@@ -264,7 +265,7 @@ gemm_bf16x3_kernel(const __grid_constant__ GemmMaps maps, int nseg, int neg_mask
       }
       tc_fence_after();
       const int r0 = tile_m * BM + 32 * quarter, n0 = tile_n * BN;
-      const int d0 = (split ? lin + (int)blockIdx.x : tile_m) * BM + 32 * quarter;  // row of D
+      const int d0 = (SPLIT ? lin + (int)blockIdx.x : tile_m) * BM + 32 * quarter;  // row of D
 #pragma unroll 1
       for (int c0 = 0; c0 < BN; c0 += 32) {
         uint32_t r[32];
@@ -338,8 +339,9 @@ cudaError_t gemm_launch(const SplitOperand* A, const SplitOperand* B, const int*
   static std::once_flag attr_once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(attr_once, [] {
-    attr_err =
-        cudaFuncSetAttribute(gemm_bf16x3_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    for (auto k : {gemm_bf16x3_kernel<BN, false>, gemm_bf16x3_kernel<BN, true>})
+      if (attr_err == cudaSuccess)
+        attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
   });
   if (attr_err != cudaSuccess) return attr_err;
   const long long tnl = (N + BN - 1) / BN, tml = (M + BM - 1) / BM;
@@ -375,8 +377,9 @@ cudaError_t gemm_launch(const SplitOperand* A, const SplitOperand* B, const int*
     frac = std::min(1.0, tn * (tn + 1) / 2.0 / (tm * tn));  // tiles with n-tile >= m-tile (tm >= tn)
   }
   ProfScope prof("gemm_bf16x3", 0.0, 6.0 * (double)M * N * K * nseg * frac, s);
-  gemm_bf16x3_kernel<BN><<<grid, GEMM_THREADS, C::SMEM_BYTES, s>>>(maps, nseg, neg_mask, M, N, K, D, ldd,
-                                                                   accumulate ? 1 : 0, err_dev, upper ? 1 : 0, split && split->ctas);
+  const auto kernel = split && split->ctas ? gemm_bf16x3_kernel<BN, true> : gemm_bf16x3_kernel<BN, false>;
+  kernel<<<grid, GEMM_THREADS, C::SMEM_BYTES, s>>>(maps, nseg, neg_mask, M, N, K, D, ldd, accumulate ? 1 : 0, err_dev,
+                                                   upper ? 1 : 0);
   return cudaGetLastError();
 }
 
