@@ -51,7 +51,8 @@ struct GemmMaps {
   CUtensorMap b[2][2];
 };
 
-constexpr int GEMM_SHARE = 4;  // fewest K blocks of a split share
+constexpr int GEMM_SHARE = 8;   // fewest K blocks of a split share
+constexpr int GEMM_SAVED = 12;  // fewest K blocks that a split takes off the longest CTA
 constexpr int GEMM_THREADS = 192;  // warp 0 loads, warp 1 issues MMAs, warps 2-5 drain accumulators
 
 // Output tile of linear index lin: groups of GROUP_M row tiles, the row tile fastest within a
@@ -361,11 +362,20 @@ cudaError_t gemm_launch(const SplitOperand* A, const SplitOperand* B, const int*
   int grid = (int)std::max(1LL, std::min<long long>(tiles, sms));
   if (split) {
     // One column tile only: with several, CTAs that work on one panel of A at the same K blocks share it in L2.
-    // A share is at least GEMM_SHARE K blocks; fewer do not pay for a CTA's start.
+    // Shares that end where their tile does cost one epilogue each and leave the reader the fewest slots, so a tile goes
+    // to k CTAs of its own where k times the tiles fill 70 % of the chip, or where k is bounded by the shortest share
+    // worth a CTA; else all CTAs take equal shares.  The slots of a short product cost more than a few K blocks.
+    // An application to 4 | 64 columns, us (whole tiles, equal shares of at least 4 K blocks, this rule): 480 functions
+    // 239, 266, 237 | 290, 314, 290; 2430: 373, 353, 332 | 454, 450, 406; 7680: 747, 625, 618 | 970, 951, 917;
+    // 30720: 6215, 4767, 4763 | 7161, 6128, 6128.
     const long long total = (long long)nseg * ((K + BK - 1) / BK), T = tiles * total;
-    const int g = (int)std::min<long long>(std::min(sms, GEMM_SLOTS), std::max(tiles, T / GEMM_SHARE));
+    const int chip = std::min(sms, GEMM_SLOTS);
+    const long long fit = chip / tiles, k = std::min(fit, total / GEMM_SHARE);
+    const bool own = k >= 2 && !(k == fit && 10 * k * tiles < 7 * chip);
+    const int g = own ? (int)(k * tiles) : fit >= 1 && total < 2 * GEMM_SHARE ? (int)tiles : chip;
     split->ctas = 0;
-    if (tnl == 1 && !accumulate && T * g < 0x7fffffffLL && tiles % g != 0) {
+    if (tnl == 1 && !accumulate && T * g < 0x7fffffffLL && tiles % g != 0 &&
+        (tiles + g - 1) / g * total - (T + g - 1) / g >= GEMM_SAVED) {
       grid = split->ctas = g;
       split->tiles = (int)tiles;
       split->total = (int)total;
