@@ -589,42 +589,41 @@ __device__ __forceinline__ void madd(double (&acc)[2 * HM_COLS], float2 e, const
   }
 }
 
-// the sums of one row (row0 + lane) of a tile over the cover entries begin + w, begin + w + step, ...
+// The sums of one row (row0 + `row`) of a tile over the cover entries begin + first, begin + first + step, ...  Each entry
+// is `count` products of a stored value (f, fs values apart) and NC columns (x, xs values apart), so that groups of
+// lanes with entries of different kinds run one loop.
 template <int NC>
 __device__ __forceinline__ void tile_rows(const HmTile& T, const int32_t* __restrict__ cover,
                                           const HmBlockDev* __restrict__ blk, const float2* __restrict__ H,
                                           const double2* __restrict__ xg, const double2* __restrict__ t, int nrhs,
-                                          int w, int step, int lane, double (&acc)[2 * HM_COLS]) {
-  const bool live = lane < T.rows;
-  for (int q = T.begin + w; q < T.end; q += step) {
+                                          int first, int step, int row, double (&acc)[2 * HM_COLS]) {
+  for (int q = T.begin + first; q < T.end; q += step) {
     const int code = cover[q];
     const HmBlockDev B = blk[code >> 1];
     const int cols = code & 1, m = B.r1 - B.r0, nn = B.c1 - B.c0;
-    const int i = T.row0 + (live ? lane : 0) - (cols ? B.c0 : B.r0);
-    const float2* M = H + B.off;
+    const int i = T.row0 + row - (cols ? B.c0 : B.r0);
+    const float2* f = H + B.off + i;
+    const double2* x = xg + (size_t)(cols ? B.r0 : B.c0) * NC;
+    int count = cols ? m : nn, fs = nn, xs = NC;
     if (B.rank >= 0) {  // U t, or Vt^T t' below the diagonal
-      const int len = cols ? nn : m;
-      const float2* f = M + (cols ? (size_t)B.rank * m : 0) + i;
-      const double2* tb = t + ((size_t)B.t0 + (cols ? B.rank : 0)) * nrhs;
-#pragma unroll 4
-      for (int l = 0; l < B.rank; ++l) madd<NC>(acc, f[(size_t)l * len], tb + (size_t)l * nrhs);
-    } else if (cols) {  // the transpose of a dense block
-      const double2* x = xg + (size_t)B.r0 * NC;
-#pragma unroll 4
-      for (int p = 0; p < m; ++p) madd<NC>(acc, M[(size_t)p * nn + i], x + (size_t)p * NC);
-    } else if (B.r0 == B.c0) {  // a diagonal block is symmetric: read it along its rows
-      const double2* x = xg + (size_t)B.c0 * NC;
-#pragma unroll 4
-      for (int j = 0; j < nn; ++j) madd<NC>(acc, M[(size_t)j * nn + i], x + (size_t)j * NC);
-    } else {
-      const double2* x = xg + (size_t)B.c0 * NC;
-#pragma unroll 4
-      for (int j = 0; j < nn; ++j) madd<NC>(acc, M[(size_t)i * nn + j], x + (size_t)j * NC);
+      if (cols) f += (size_t)B.rank * m;
+      else fs = m;
+      x = t + ((size_t)B.t0 + (cols ? B.rank : 0)) * nrhs;
+      count = B.rank;
+      xs = nrhs;
+    } else if (!cols && B.r0 != B.c0) {  // along a row; a diagonal block is symmetric, a transposed one lies so
+      f += (size_t)i * (nn - 1);
+      fs = 1;
     }
+#pragma unroll 4
+    for (int l = 0; l < count; ++l, f += fs, x += xs) madd<NC>(acc, *f, x);
   }
 }
 
 // A cluster of CTAs per tile and group, the cover entries dealt to all their warps; the first adds their sums in order.
+// Where a tile has at most 16 or 8 rows (small leaves) and more entries than warps, a warp takes two or four entries at
+// a time, one per 16 or 8 lanes: leaves of 8, both products of 14520 functions and 9680 cells, one column, 3.4 ms
+// with an entry a warp and 1.5 so.
 __global__ void __launch_bounds__(HM_THREADS)
     hm_rows_kernel(const HmTile* __restrict__ tiles, const int32_t* __restrict__ cover,
                    const HmBlockDev* __restrict__ blk, const float2* __restrict__ H, const double2* __restrict__ xp,
@@ -639,15 +638,18 @@ __global__ void __launch_bounds__(HM_THREADS)
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = blockIdx.y * HM_COLS, nc = min(HM_COLS, nrhs - g);
   const double2* xg = xp + (size_t)g * n;
-  const int first = w * team + rank, step = HM_ROW_WARPS * team;
+  const bool many = T.end - T.begin > HM_ROW_WARPS * team;
+  const int R = many && T.rows <= 8 ? 8 : (many && T.rows <= 16 ? 16 : HM_TILE), subs = HM_TILE / R;  // lanes of an entry
+  const int first = (w * team + rank) * subs + lane / R, step = HM_ROW_WARPS * team * subs;
+  const int row = lane % R < T.rows ? lane % R : 0;
   double acc[2 * HM_COLS];
 #pragma unroll
   for (int k = 0; k < 2 * HM_COLS; ++k) acc[k] = 0.0;
   switch (nc) {
-    case 1: tile_rows<1>(T, cover, blk, H, xg, t + g, nrhs, first, step, lane, acc); break;
-    case 2: tile_rows<2>(T, cover, blk, H, xg, t + g, nrhs, first, step, lane, acc); break;
-    case 3: tile_rows<3>(T, cover, blk, H, xg, t + g, nrhs, first, step, lane, acc); break;
-    default: tile_rows<4>(T, cover, blk, H, xg, t + g, nrhs, first, step, lane, acc); break;
+    case 1: tile_rows<1>(T, cover, blk, H, xg, t + g, nrhs, first, step, row, acc); break;
+    case 2: tile_rows<2>(T, cover, blk, H, xg, t + g, nrhs, first, step, row, acc); break;
+    case 3: tile_rows<3>(T, cover, blk, H, xg, t + g, nrhs, first, step, row, acc); break;
+    default: tile_rows<4>(T, cover, blk, H, xg, t + g, nrhs, first, step, row, acc); break;
   }
 #pragma unroll
   for (int k = 0; k < 2 * HM_COLS; ++k) part[w][k][lane] = acc[k];
@@ -657,6 +659,9 @@ __global__ void __launch_bounds__(HM_THREADS)
   double s = 0.0;
 #pragma unroll
   for (int v = 0; v < HM_ROW_WARPS; ++v) s += part[v][k][i];
+  for (int z = i + R; i < R && z < HM_TILE; z += R)  // the other entries of the warps
+#pragma unroll
+    for (int v = 0; v < HM_ROW_WARPS; ++v) s += part[v][k][z];
   if (team > 1) {
     sums[threadIdx.x] = s;
     cl.sync();
@@ -674,9 +679,11 @@ __global__ void __launch_bounds__(HM_THREADS)
 // cells, both products of one and of four columns 128 and 302 us with one CTA a tile, 77 and 151 so; 18000
 // functions and 12000 cells, one column 1.09 and 1.03 ms.  Cutting the entries into pieces of 16 or 32 terms as
 // well gave nothing.
-int hm_team(long long ctas) {
+// CTAs beyond the entries of every tile would have no work (225 functions in four blocks a row, 40 columns: 90 us with 8
+// CTAs a tile, 49 with 4).
+int hm_team(long long ctas, int entries) {
   int team = 1;
-  while (team < 8 && ctas * team < 4 * 152) team *= 2;
+  while (team < 8 && ctas * team < 4 * 152 && team < entries) team *= 2;
   return team;
 }
 
@@ -692,7 +699,7 @@ struct HmPart {
   int2* items = nullptr;         // cross items of the low-rank blocks, longest first (device)
   HmTile* tiles = nullptr;       // row tiles (device)
   int32_t* cover = nullptr;      // blocks over each tile (device)
-  int nitems = 0, ntiles = 0, ncross = 0;
+  int nitems = 0, ntiles = 0, entries = 0, ncross = 0;  // entries: most over one tile
   long long elems = 0;
   int64_t n_lowrank = 0, n_dense = 0, n_capped = 0, n_small = 0;
   int max_rank = 0;
@@ -935,6 +942,7 @@ int finish_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, PartBuil
   HM_CUDA(cudaStreamSynchronize(0));  // packed, and the pool has the temporaries back
   out.nitems = (int)items.size();
   out.ntiles = (int)lists.tiles.size();
+  for (const HmTile& t : lists.tiles) out.entries = std::max(out.entries, t.end - t.begin);
   HM_CUDA(keep(&out.items, items, owned));
   HM_CUDA(keep(&out.tiles, lists.tiles, owned));
   HM_CUDA(keep(&out.cover, lists.cover, owned));
@@ -1140,7 +1148,7 @@ int rfcmp_hm_apply(rfcmp_hm* hm, int which, const rfcmp_c128* x, rfcmp_c128* y, 
       hm_cross_kernel<<<dim3((P.nitems + per - 1) / per, groups), HM_CROSS_THREADS, 0, st>>>(
           P.blocks, P.items, P.nitems, P.data, xp, t, P.n, nr);
     }
-    const int team = hm_team((long long)P.ntiles * groups);
+    const int team = hm_team((long long)P.ntiles * groups, P.entries);
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = (unsigned)team;
