@@ -789,15 +789,6 @@ std::vector<int2> cross_items(const std::vector<HmBlockDev>& blk) {
   return items;
 }
 
-template <class T>
-cudaError_t keep(T** d, const std::vector<T>& h, std::vector<void*>& owned) {
-  if (h.empty()) return cudaSuccess;
-  cudaError_t e = dev_malloc(d, h.size() * sizeof(T));
-  if (e != cudaSuccess) return e;
-  owned.push_back(*d);
-  return cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
-}
-
 // One matrix on its way to the compressed form: the partition (host), the cross approximations (queued
 // on the legacy stream) and what the packing reads.
 struct PartBuild {
@@ -837,9 +828,9 @@ int start_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, uint64_t 
     // the blocks and, beside them, first the slots and lists of the approximations, then the lists of the product
     b.lists = cover_lists(b.blocks, n);
     const uint64_t nb = b.blocks.size(), nc = b.cand.size();
-    const uint64_t temps = 8ull * (uint64_t)slot_elems + nc * (sizeof(HmBlockDev) + 20) + 8 * nb;
+    const uint64_t temps = 8ull * (uint64_t)slot_elems + nc * (sizeof(HmBlockDev) + 20);
     const uint64_t keeps = item_bytes + sizeof(HmTile) * b.lists.tiles.size() + 4ull * b.lists.cover.size();
-    const uint64_t peak = 8ull * (uint64_t)worst + sizeof(HmBlockDev) * nb + 4ull * n + std::max(temps, keeps);
+    const uint64_t peak = 8ull * (uint64_t)worst + (sizeof(HmBlockDev) + 8) * nb + 4ull * n + std::max(temps, keeps);
     if (peak > budget_left)
       return set_error(RFCMP_ERR_OUT_OF_BUDGET, "compression needs up to " + std::to_string(peak) +
                                                     " bytes, budget has " + std::to_string(budget_left));
@@ -927,14 +918,18 @@ int finish_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, PartBuil
   out.nblocks = (int)fin.size();
   HM_CUDA(dev_malloc(&out.data, std::max<size_t>(8 * (size_t)off, 8)));
   owned.push_back(out.data);
-  HM_CUDA(dev_malloc(&out.blocks, std::max<size_t>(fin.size() * sizeof(HmBlockDev), 8)));
-  owned.push_back(out.blocks);
   if (!fin.empty()) {
-    long long* fslot_d = nullptr;
-    HM_CUDA(b.tmp.alloc(&fslot_d, fin_slot.size() * sizeof(long long)));
-    HM_CUDA(cudaMemcpy(out.blocks, fin.data(), fin.size() * sizeof(HmBlockDev), cudaMemcpyHostToDevice));
-    HM_CUDA(cudaMemcpy(fslot_d, fin_slot.data(), fin_slot.size() * sizeof(long long), cudaMemcpyHostToDevice));
-    hm_pack_kernel<<<(unsigned)fin.size(), HM_THREADS>>>(A, ld, out.perm, out.blocks, fslot_d, cap, b.slots, out.data);
+    const size_t nb = fin.size(), at = nb * sizeof(HmBlockDev);
+    std::vector<char> buf(at + 8 * nb);  // the blocks, then their slots
+    std::memcpy(buf.data(), fin.data(), at);
+    std::memcpy(buf.data() + at, fin_slot.data(), 8 * nb);
+    char* d = nullptr;
+    HM_CUDA(dev_malloc(&d, buf.size()));
+    owned.push_back(d);
+    HM_CUDA(cudaMemcpy(d, buf.data(), buf.size(), cudaMemcpyHostToDevice));
+    out.blocks = reinterpret_cast<HmBlockDev*>(d);
+    hm_pack_kernel<<<(unsigned)nb, HM_THREADS>>>(A, ld, out.perm, out.blocks, reinterpret_cast<long long*>(d + at), cap,
+                                                 b.slots, out.data);
     HM_CUDA(cudaGetLastError());
   }
   const std::vector<int2> items = cross_items(fin);
@@ -943,10 +938,22 @@ int finish_part(const float2* A, int ld, int n, const rfcmp_hm_opts& o, PartBuil
   out.nitems = (int)items.size();
   out.ntiles = (int)lists.tiles.size();
   for (const HmTile& t : lists.tiles) out.entries = std::max(out.entries, t.end - t.begin);
-  HM_CUDA(keep(&out.items, items, owned));
-  HM_CUDA(keep(&out.tiles, lists.tiles, owned));
-  HM_CUDA(keep(&out.cover, lists.cover, owned));
-  out.bytes = 8ull * (uint64_t)off + sizeof(HmBlockDev) * fin.size() + 4ull * n + sizeof(int2) * items.size() +
+  // the product's lists in one buffer (an upload each took as long as the rest of a small body's compression)
+  const size_t at_tiles = sizeof(int2) * items.size(), at_cover = at_tiles + sizeof(HmTile) * lists.tiles.size();
+  std::vector<char> buf(at_cover + 4 * lists.cover.size());
+  if (!buf.empty()) {
+    if (!items.empty()) std::memcpy(buf.data(), items.data(), at_tiles);
+    std::memcpy(buf.data() + at_tiles, lists.tiles.data(), at_cover - at_tiles);
+    std::memcpy(buf.data() + at_cover, lists.cover.data(), buf.size() - at_cover);
+    char* d = nullptr;
+    HM_CUDA(dev_malloc(&d, buf.size()));
+    owned.push_back(d);
+    HM_CUDA(cudaMemcpy(d, buf.data(), buf.size(), cudaMemcpyHostToDevice));
+    out.items = reinterpret_cast<int2*>(d);
+    out.tiles = reinterpret_cast<HmTile*>(d + at_tiles);
+    out.cover = reinterpret_cast<int32_t*>(d + at_cover);
+  }
+  out.bytes = 8ull * (uint64_t)off + (sizeof(HmBlockDev) + 8) * fin.size() + 4ull * n + sizeof(int2) * items.size() +
               sizeof(HmTile) * lists.tiles.size() + 4ull * lists.cover.size();
   return RFCMP_OK;
 }
@@ -1075,12 +1082,12 @@ int rfcmp_hm_create(rfcmp_op* op, const rfcmp_hm_opts* opts_in, rfcmp_hm** out) 
     const float2* mats[2] = {v.TA, v.V};
     const int lds[2] = {v.ldN, v.ldC}, ns[2] = {v.n, v.nc};
     PartBuild part[2];
-    // the host partitions V beside T_A (a thread of its own, or after it where none can be had); the builds
-    // follow one another, so that the peak is one matrix's slots
+    // the host partitions V beside T_A (a thread of its own, or after it where none can be had or V's partition takes
+    // no longer than to start one); the builds follow one another, so that the peak is one matrix's slots
     auto split_v = [&] { partition(ccen.data(), clo.data(), chi.data(), v.nc, o.leaf, o.eta, part[1].perm, part[1].blocks); };
     std::future<void> other;
     try {
-      other = std::async(std::launch::async, split_v);
+      if (v.nc >= 12 * o.leaf) other = std::async(std::launch::async, split_v);
     } catch (const std::system_error&) {
     }
     partition(ecen.data(), elo.data(), ehi.data(), v.n, o.leaf, o.eta, part[0].perm, part[0].blocks);
