@@ -2748,16 +2748,20 @@ int rfcmp_farfield(rfcmp_op* op, const rfcmp_c128* j, int64_t nrhs, const double
   if (!op || !j || !dirs || !rcs_dbsm || nrhs <= 0 || ndir <= 0 || nrhs > 65535 || ndir > (1 << 20))
     return set_error(RFCMP_ERR_INVALID_ARG, "invalid argument");
   cudaStream_t st = (cudaStream_t)stream;
-  double* dd = nullptr;
-  double2* dn = nullptr;
-  RF_CUDA(cudaMallocAsync(&dd, sizeof(double) * 3 * ndir, st));
-  RF_CUDA(cudaMallocAsync(&dn, sizeof(double2) * 3 * ndir * nrhs, st));
-  RF_CUDA(cudaMemcpyAsync(dd, dirs, sizeof(double) * 3 * ndir, cudaMemcpyHostToDevice, st));
-  RF_K(launch_farfield(op->g, op->k, reinterpret_cast<const double2*>(j), (int)nrhs, dd, (int)ndir, dn, st));
-  std::vector<double2> h(3 * ndir * nrhs);
-  RF_CUDA(cudaMemcpyAsync(h.data(), dn, sizeof(double2) * h.size(), cudaMemcpyDeviceToHost, st));
-  RF_CUDA(cudaFreeAsync(dd, st));
-  RF_CUDA(cudaFreeAsync(dn, st));
+  // the radiation vectors, the directions and the scratch of the kernels in one buffer
+  const size_t vec = 6 * (size_t)ndir * nrhs, dir = (3 * (size_t)ndir + 1) / 2 * 2;
+  double* buf = nullptr;
+  RF_CUDA(cudaMallocAsync(&buf, sizeof(double) * (vec + dir + farfield_scratch((int)op->g.nc, (int)nrhs, (int)ndir)), st));
+  double *dn = buf, *dd = buf + vec;
+  cudaError_t err = cudaMemcpyAsync(dd, dirs, sizeof(double) * 3 * ndir, cudaMemcpyHostToDevice, st);
+  if (err == cudaSuccess)
+    err = launch_farfield(op->g, op->k, reinterpret_cast<const double2*>(j), (int)nrhs, dd, (int)ndir,
+                          reinterpret_cast<double2*>(dn), dd + dir, st);
+  std::vector<double2> h(3 * ndir * nrhs);  // beside the kernels
+  if (err == cudaSuccess) err = cudaMemcpyAsync(h.data(), dn, sizeof(double2) * h.size(), cudaMemcpyDeviceToHost, st);
+  const cudaError_t freed = cudaFreeAsync(buf, st);
+  RF_CUDA(err);
+  RF_CUDA(freed);
   RF_CUDA(cudaStreamSynchronize(st));
   const double k = op->k;
   for (int64_t r = 0; r < nrhs; ++r)

@@ -18,6 +18,7 @@
 // the second by the 7-point rule; the result is the mean of both orders.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "rfcmp_internal.h"
@@ -674,7 +675,8 @@ __global__ void rhs_kernel(const DeviceGeometry g, double k, const double* __res
 // GB300: 362 directions of one current on 20480 cells 5.10 -> 1.98 ms (the FP64 floor of 138 operations
 // is 1.63 ms); 91 directions of 23 currents on 1600 cells 1.11 -> 0.46 ms.
 constexpr int FF_THREADS = 128;
-constexpr int FF_COLS = 64;  // right-hand sides of one pass (bounds the cell currents' scratch)
+constexpr int FF_COLS = 64;  // right-hand sides of one pass, more where their cell currents' scratch fits FF_SCRATCH
+constexpr size_t FF_SCRATCH = (size_t)256 << 20;
 
 // cos and sin of |x| <= 1/2 by their Taylor series (to x^12 and x^13: truncation below 1e-15)
 __device__ __forceinline__ void sincos_small64(double x, double* s, double* c) {
@@ -973,37 +975,55 @@ cudaError_t launch_rhs_planewave(const DeviceGeometry& g, double k, const double
   return cudaGetLastError();
 }
 
-cudaError_t launch_farfield(const DeviceGeometry& g, double k, const double2* j, int nrhs, const double* dirs,
-                            int ndir, double2* out, cudaStream_t s) {
-  ProfScope prof("farfield", 0.0, 0.0, s);
-  const int cols = nrhs < FF_COLS ? nrhs : FF_COLS;
-  // eight right-hand sides share B0 and B1 where there are that many (48 sums a thread); a chunk is as
-  // many blocks of 128 cells as leave twelve CTAs a SM, at least two so that the sums over the CTA
-  // (about a fifth of one block's work) stay small
-  const int rb = cols == 1 ? 1 : (cols <= 4 ? 4 : 8);
-  const long long groups = (cols + rb - 1) / rb, nb = (g.nc + FF_THREADS - 1) / FF_THREADS;
+namespace {
+struct FarPlan {
+  int cols, rb, bpc, chunks;  // right-hand sides of a pass and of a CTA, blocks of 128 cells of a chunk, chunks
+  size_t geo, cur, part;      // doubles of scratch: cell geometry, cell currents, partial sums
+};
+FarPlan far_plan(int nc, int nrhs, int ndir) {
+  FarPlan p;
+  p.cols = std::min(nrhs, std::max(FF_COLS, (int)std::min<size_t>(FF_SCRATCH / (64 * (size_t)nc) / 8 * 8, 65528)));
+  // eight right-hand sides share B0 and B1 where there are that many (48 sums a thread); a chunk is as many blocks
+  // of 128 cells as make twelve CTAs a SM (four are resident with one right-hand side, two with 4 or 8, whose
+  // 242 and 255 registers a thread fill the SM; eight also spill 216 bytes), at least two so that the sums over the
+  // CTA (about a fifth of one block's work) stay small
+  p.rb = p.cols == 1 ? 1 : (p.cols <= 4 ? 4 : 8);
+  const long long groups = (p.cols + p.rb - 1) / p.rb, nb = (nc + FF_THREADS - 1) / FF_THREADS;
   const long long per = (nb * groups * ndir) / (152 * 12);
-  const int bpc = (int)(per < 2 ? 2 : (per > nb ? nb : per));
-  const int chunks = (int)((nb + bpc - 1) / bpc);
-  double* buf = nullptr;
-  const size_t geo = (size_t)9 * g.nc, cur = (size_t)8 * cols * g.nc, part = (size_t)chunks * cols * ndir * 6;
-  cudaError_t e = cudaMallocAsync(&buf, sizeof(double) * (geo + cur + part), s);
-  if (e != cudaSuccess) return e;
-  double *pcur = buf + geo, *ppart = pcur + cur;
-  for (int r = 0; r < nrhs && e == cudaSuccess; r += cols) {
-    const int nr = nrhs - r < cols ? nrhs - r : cols;
-    farfield_cells_kernel<<<dim3((g.nc + 127) / 128, nr), 128, 0, s>>>(g, k, j + (size_t)r * g.ne, nr, buf, pcur);
-    const dim3 grid(ndir, (nr + rb - 1) / rb, chunks);
-    if (rb == 1) farfield_kernel<1><<<grid, FF_THREADS, 0, s>>>(g.nc, buf, pcur, nr, dirs, ndir, bpc, ppart);
-    else if (rb == 4) farfield_kernel<4><<<grid, FF_THREADS, 0, s>>>(g.nc, buf, pcur, nr, dirs, ndir, bpc, ppart);
-    else farfield_kernel<8><<<grid, FF_THREADS, 0, s>>>(g.nc, buf, pcur, nr, dirs, ndir, bpc, ppart);
+  p.bpc = (int)(per < 2 ? 2 : (per > nb ? nb : per));
+  p.chunks = (int)((nb + p.bpc - 1) / p.bpc);
+  p.geo = (size_t)9 * nc;
+  p.cur = (size_t)8 * p.cols * nc;
+  p.part = p.chunks > 1 ? (size_t)p.chunks * p.cols * ndir * 6 : 0;  // one chunk: straight to the result
+  return p;
+}
+}  // namespace
+
+size_t farfield_scratch(int nc, int nrhs, int ndir) {
+  const FarPlan p = far_plan(nc, nrhs, ndir);
+  return p.geo + p.cur + p.part;
+}
+
+cudaError_t launch_farfield(const DeviceGeometry& g, double k, const double2* j, int nrhs, const double* dirs,
+                            int ndir, double2* out, double* scratch, cudaStream_t s) {
+  ProfScope prof("farfield", 0.0, 0.0, s);
+  const FarPlan p = far_plan(g.nc, nrhs, ndir);
+  double *geo = scratch, *cur = geo + p.geo;
+  cudaError_t e = cudaSuccess;
+  for (int r = 0; r < nrhs && e == cudaSuccess; r += p.cols) {
+    const int nr = std::min(nrhs - r, p.cols);
+    double* o = reinterpret_cast<double*>(out + (size_t)r * ndir * 3);
+    double* part = p.chunks > 1 ? cur + p.cur : o;
+    farfield_cells_kernel<<<dim3((g.nc + 127) / 128, nr), 128, 0, s>>>(g, k, j + (size_t)r * g.ne, nr, geo, cur);
+    const dim3 grid(ndir, (nr + p.rb - 1) / p.rb, p.chunks);
+    if (p.rb == 1) farfield_kernel<1><<<grid, FF_THREADS, 0, s>>>(g.nc, geo, cur, nr, dirs, ndir, p.bpc, part);
+    else if (p.rb == 4) farfield_kernel<4><<<grid, FF_THREADS, 0, s>>>(g.nc, geo, cur, nr, dirs, ndir, p.bpc, part);
+    else farfield_kernel<8><<<grid, FF_THREADS, 0, s>>>(g.nc, geo, cur, nr, dirs, ndir, p.bpc, part);
     const long long n = (long long)nr * ndir * 6;
-    farfield_sum_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(ppart, chunks, n,
-                                                                   reinterpret_cast<double*>(out + (size_t)r * ndir * 3));
+    if (p.chunks > 1) farfield_sum_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(part, p.chunks, n, o);
     e = cudaGetLastError();
   }
-  const cudaError_t f = cudaFreeAsync(buf, s);
-  return e != cudaSuccess ? e : f;
+  return e;
 }
 
 RF_LAUNCH_READER(launches_assembly)

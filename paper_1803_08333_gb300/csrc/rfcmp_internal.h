@@ -182,8 +182,9 @@ cudaError_t launch_rhs_voltage_gap(const DeviceGeometry& g, const double* origin
 cudaError_t launch_rhs_planewave(const DeviceGeometry& g, double k, const double* khat, const double* pol,
                                  int nrhs, double2* e, cudaStream_t s);
 // radiation vector N(rhat) for nrhs currents and ndir directions -> out (ndir x nrhs x 3 complex)
-cudaError_t launch_farfield(const DeviceGeometry& g, double k, const double2* j, int nrhs, const double* dirs,
-                            int ndir, double2* out, cudaStream_t s);
+cudaError_t launch_farfield(const DeviceGeometry& g, double k, const double2* j, int nrhs, const double* dirs, int ndir,
+                            double2* out, double* scratch, cudaStream_t s);
+size_t farfield_scratch(int nc, int nrhs, int ndir);  // doubles
 
 // ---------------------------------------------------------------- tensor-core GEMM (k_gemm.cu)
 // A BF16 operand split in two planes (hi = bf16(x), lo = bf16(x - hi)), row-major with K
