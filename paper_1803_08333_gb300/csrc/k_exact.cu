@@ -332,20 +332,22 @@ __global__ void __launch_bounds__(DT) digits_kernel(Src src, int K, long long ld
   }
 }
 
-// Re and Im of one column of X per cluster of XCL CTAs: each takes a slice of K, the column maxima
+// Re and Im of one column of X per cluster of CTAs: each takes a slice of K, the column maxima
 // meet through distributed shared memory, then every slice writes its digits.  Rows 0..nr-1 of the
-// planes are Re of the columns, rows nr..2nr-1 Im.
+// planes are Re of the columns, rows nr..2nr-1 Im.  Up to XCL CTAs of at least XCL_PAIRS
+// pairs of entries: a cluster of 8 costs a body of 120 functions 7 us a product more (64 columns, 57 and 64 us).
 constexpr int XCL = 8;
-__global__ void __cluster_dims__(XCL, 1, 1) __launch_bounds__(DT)
+constexpr int XCL_PAIRS = 64;
+__global__ void __launch_bounds__(DT)
 x_digits_kernel(const double2* __restrict__ X, int n, int nr, long long ldp, uint32_t* __restrict__ planes,
                 int* __restrict__ e_out) {
   RF_COUNT_LAUNCH();
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   __shared__ unsigned long long mx[2];
-  const int r = blockIdx.y, rank = (int)cl.block_rank();
+  const int r = blockIdx.y, rank = (int)cl.block_rank(), team = (int)cl.num_blocks();
   const double2* x = X + (size_t)r * n;
-  const int pairs = (int)(ldp / 2), p0 = (int)((long long)pairs * rank / XCL), p1 = (int)((long long)pairs * (rank + 1) / XCL);
+  const int pairs = (int)(ldp / 2), p0 = (int)((long long)pairs * rank / team), p1 = (int)((long long)pairs * (rank + 1) / team);
   if (threadIdx.x < 2) mx[threadIdx.x] = 0;
   __syncthreads();
   unsigned long long a = 0, b = 0;
@@ -367,7 +369,7 @@ x_digits_kernel(const double2* __restrict__ X, int n, int nr, long long ldp, uin
 #pragma unroll
   for (int z = 0; z < 2; ++z) {
     unsigned long long m = 0;
-    for (int c = 0; c < XCL; ++c) m = max(m, *cl.map_shared_rank(&mx[z], c));
+    for (int c = 0; c < team; ++c) m = max(m, *cl.map_shared_rank(&mx[z], c));
     e[z] = m == 0 ? 0 : (m >> 52) == 2047 ? NOT_FINITE : ilogb(__longlong_as_double((long long)m)) + 2;
     if (rank == 0 && threadIdx.x == 0) e_out[z * nr + r] = e[z];
   }
@@ -386,14 +388,17 @@ x_digits_kernel(const double2* __restrict__ X, int n, int nr, long long ldp, uin
 }
 
 // Y[:, r] = scale * op(T) X[:, r] (+ Y) from the integer sums of [Tr; Ti] [Xr Xi] or (real) P [Xr Xi],
-// at most XI_COLS columns: a CTA reads 32 rows of D along their columns and writes Y along its rows
+// at most XI_COLS columns: a CTA reads R rows of D along their columns and writes Y along its rows.
+// The FP64 pipe takes 8 us for 32 rows of 32 columns, so small matrices take 8 rows a CTA (COMBINE_SMALL).
 constexpr int XI_COLS = 32;
+constexpr int COMBINE_SMALL = 32 * 152;
+template <int R>
 __global__ void __launch_bounds__(DT)
 combine_int_kernel(const longlong2* __restrict__ D, const int* __restrict__ ea, const int* __restrict__ eb, int n,
                    int nr, int conj, int real, double2 scale, int accumulate, double2* __restrict__ Y) {
   RF_COUNT_LAUNCH();
-  __shared__ double2 t[XI_COLS][33];
-  const int i0 = blockIdx.x * 32;
+  __shared__ double2 t[XI_COLS][R + 1];
+  const int i0 = blockIdx.x * R;
   auto value = [&](int row, int col) {
     const longlong2 d = D[(size_t)row * (2 * nr) + col];
     const int x = eb[col];
@@ -402,7 +407,7 @@ combine_int_kernel(const longlong2* __restrict__ D, const int* __restrict__ ea, 
     return ldexp((double)d.x, e - 32) + ldexp((double)d.y, e - 56);
   };
   const double sg = conj ? -1.0 : 1.0;
-  for (int q = threadIdx.x; q < 32 * nr; q += DT) {
+  for (int q = threadIdx.x; q < R * nr; q += DT) {
     const int i = i0 + q / nr, r = q % nr;
     if (i >= n) break;
     double2 v = make_double2(value(i, r), value(i, nr + r));
@@ -413,10 +418,10 @@ combine_int_kernel(const longlong2* __restrict__ D, const int* __restrict__ ea, 
     t[r][i - i0] = make_double2(scale.x * v.x - scale.y * v.y, scale.x * v.y + scale.y * v.x);
   }
   __syncthreads();
-  for (int q = threadIdx.x; q < 32 * nr; q += DT) {
-    const int r = q >> 5, i = i0 + (q & 31);
+  for (int q = threadIdx.x; q < R * nr; q += DT) {
+    const int r = q / R, i = i0 + q % R;
     if (i >= n) continue;
-    double2 o = t[r][q & 31];
+    double2 o = t[r][q % R];
     double2* y = Y + (size_t)r * n + i;
     if (accumulate) {
       o.x += y->x;
@@ -524,15 +529,29 @@ cudaError_t exact_product(const ExactOperand& T, int n, const double2* X, double
   B.rows = 2 * nr;
   B.ldp = T.ldp;
   B.plane_stride = (long long)2 * nr * T.ldp;
-  x_digits_kernel<<<dim3(XCL, nr), DT, 0, s>>>(X, n, nr, B.ldp, reinterpret_cast<uint32_t*>(B.d), B.e);
-  cudaError_t e = cudaGetLastError();
+  int team = 1;
+  while (team < XCL && 2LL * team * XCL_PAIRS <= B.ldp / 2) team *= 2;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)team;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)team, (unsigned)nr);
+  cfg.blockDim = dim3(DT);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = team > 1 ? 1 : 0;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, x_digits_kernel, X, n, nr, (long long)B.ldp, reinterpret_cast<uint32_t*>(B.d), B.e);
   if (e != cudaSuccess) return e;
   const bool ints = nr <= XI_COLS;
   longlong2* DI = ints ? reinterpret_cast<longlong2*>(w.D64) : nullptr;
   if ((e = exact_gemm(T, B, rows, 2 * nr, n, w.D64, DI, 2 * nr, w.err, s)) != cudaSuccess) return e;
   if (ints) {
-    combine_int_kernel<<<(n + 31) / 32, DT, 0, s>>>(DI, T.e, B.e, n, nr, conj ? 1 : 0, real ? 1 : 0, scale,
-                                                   accumulate ? 1 : 0, Y);
+    auto combine = [&](auto kernel, int R) {
+      kernel<<<(n + R - 1) / R, DT, 0, s>>>(DI, T.e, B.e, n, nr, conj ? 1 : 0, real ? 1 : 0, scale, accumulate ? 1 : 0, Y);
+    };
+    if (n < COMBINE_SMALL) combine(combine_int_kernel<8>, 8);
+    else combine(combine_int_kernel<32>, 32);
   } else {
     const dim3 g((n + CT - 1) / CT, (nr + CT - 1) / CT), b(CT, 8);
     combine_f64_kernel<<<g, b, 0, s>>>(w.D64, 2 * nr, n, nr, conj ? 1 : 0, real ? 1 : 0, scale, accumulate ? 1 : 0, Y);
