@@ -271,9 +271,13 @@ constexpr int NS_MIN_CELLS = 256;
 // GEMV's pass per 4 columns (measured on GB300 from 2k to 31k unknowns).
 constexpr int MRHS_MIN = 4;
 // Float-float accurate products (right-hand side, refinement residuals, accurate applications)
-// with at least this many columns run as exact-digit tensor-core products instead of the
-// float-float GEMV, which spends some 40 FP32 instructions per complex multiply-add (measured on
-// GB300: the exact-digit product wins from 4 columns at 2k unknowns, from 2 at 17k and above).
+// with at least this many columns run as exact-digit tensor-core products, one pass for up to 32
+// columns, instead of the float-float GEMVs.  GB300, us, float-float for 1, 2, 3, 4 columns | digits for up to 4: T_A
+// of 480 functions 21, 19, 26, 20 | 55; 1920: 20, 37, 57, 59 | 65; 7680: 107, 279, 381, 533 | 283; 30720: 1456,
+// 3656, 5119, 7248 | 3390; (Sigma^T Sigma)^+ of 5120 cells 62, 102, 153, 181 | 89; 20480: 538, 1025, 1555, 1998 | 810.
+// So blocks of 4 columns are even at 2000 functions and twice as fast from 5000 on (smaller bodies lose some 30 us
+// a product).  2 and 3 columns of large bodies would gain as well, but the digits take 24 bytes an entry of T_A and
+// V beside its 8 and a pass to form.
 constexpr int EXACT_MIN = 4;
 constexpr double NS_START_TOL = 1e-2;
 constexpr int NS_MAX_STEPS = 24;

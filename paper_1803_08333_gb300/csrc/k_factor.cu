@@ -75,11 +75,13 @@ ns_residual_kernel(const double* __restrict__ X, long long ldx, int n, const int
 // L has the cell's neighbour count on its diagonal and -1 per neighbour (at most three), so a row of X M
 // is a sum of X entries: X is taken as integers of 2^(e - 60) (|X| < 2^(e - 1), e from the largest
 // diagonal entry, which bounds a positive definite matrix), the row is staged in shared memory, and the
-// sums and 1 / alpha - (X M)_ij are exact 64-bit integers; the integer rounding of an entry is 2^-8 of
-// FP64's at the top of the range.  The row's sum for the 1 1^T / n term and the BF16 split of X, which
-// the product after this reads, come out of the same pass (they took a pass over X each).  Bound: the
-// integer pipe (62 % busy) and DRAM, 16 bytes an entry (8 read, 4 + 4 written; 34 %); the FP64 form was
-// bound by the FP64 pipe.  8000 cells on GB300: 0.87 ms for the three passes, 0.36 ms in this one.
+// sums and 1 / alpha - (X M)_ij are exact 64-bit integers.  An entry of at least 2^-6 of the largest diagonal's power
+// of two converts exactly; a smaller one is rounded at 2^-59 of that power and so keeps fewer than FP64's 53 bits,
+// with an absolute error below that of an FP64 sum beside a diagonal entry.  The row's sum for the 1 1^T / n term and
+// the BF16 split of X, which the product after this reads, come out of the same pass (they took a pass over X each).
+// Bound: the conversions and the integer sums (at 5120 cells the FP64 pipe, which converts 64-bit integers, 60 % busy,
+// the integer pipe 52 %) beside DRAM, 16 bytes an entry (8 read, 4 + 4 written; 26 %); the FP64 form was bound by the
+// FP64 pipe alone (90 %).  8000 cells on GB300: 0.87 ms for the three passes, 0.36 ms in this one.
 // Rows longer than LAP_MAX do not fit shared memory and take the kernels around this one.
 constexpr int LAP_MAX = 28900;
 constexpr int FIX_BITS = 60;

@@ -4,15 +4,17 @@
 // The operator products of a single-right-hand-side solve are HBM bound: each application
 // streams T_A, V and the factors once.  A register-pipelined GEMV keeps only as many bytes in
 // flight as its unrolled loads allow; here one producer thread per CTA issues cp.async.bulk
-// copies of whole row segments (8 rows x 512 complex64 or 1024 FP32 values, 32 KB per stage)
-// together with the matching segment of x into shared-memory rings of four to six stages per SM
-// (one CTA with four stages, or two CTAs with two or three where the registers allow twice the
-// warps), so 128 to 192 KB of matrix per SM are in flight whatever the consumers do; consumers read the matrix and x from
-// shared memory only and release a stage through an mbarrier.  Three kernels:
+// copies of whole row segments together with the matching part of x into a shared-memory ring, so that
+// 128 to 192 KB of matrix per SM are in flight whatever the consumers do; consumers release a stage through an
+// mbarrier.  Three kernels:
 //   * gemv_sym_kernel (FP32 mode, symmetric M: T_A, V and the factors): reads only the tiles on
-//     and above the diagonal and forms both the row and the mirrored column product;
-//   * gemv_sym_ff_kernel (float-float, symmetric M): the accurate products, from the same tiles;
-//   * gemv_stream_ff_kernel (float-float, one column of a complex64 M): one consumer warp per row of a stage.
+//     and above the diagonal and forms both the row and the mirrored column product.  A stage is 8 rows x 512
+//     complex64 or 1024 FP32 values (32 KB) and x of the segment; one CTA with four stages, or two CTAs with two or
+//     three where the registers allow twice the warps;
+//   * gemv_sym_ff_kernel (float-float, symmetric M): the accurate products, from 32 KB tiles of 8 rows of complex
+//     values or 4 rows of hi and lo ones, three stages, two CTAs (FfStage);
+//   * gemv_stream_ff_kernel (float-float, one column of a complex64 M): one consumer warp per row of a stage of 8
+//     rows x 704 values (44 KB) and x hi and lo, two stages, two CTAs (FF_ROW, FF_NST).
 // Work units are dealt to persistent CTAs in contiguous ranges of equal size; partial sums meet
 // in FP64 atomics.  Every wait is bounded and records an error code on timeout.
 #include <cuda_runtime.h>

@@ -200,7 +200,7 @@ struct SplitOperand {
 // bounded device-side wait gave up.
 // bn selects the N tile (32, 64 or 128); 0 picks it from N.  With upper, only the 128 x 128 tiles
 // on or above the diagonal are computed (for a result known to be symmetric).
-// With split (N within one tile): the K blocks of all row tiles may be dealt to the CTAs in equal shares, which
+// With split (N within one tile): the K blocks of all row tiles may be dealt to the CTAs in shares, which
 // writes *split with ctas > 0 and D as tile slots of 128 rows (GEMM_SLOTS more than the tiles), the sum of
 // a tile by CTA b in slot tile + b.
 constexpr int GEMM_SLOTS = 160;  // bound on the CTAs of a split product
