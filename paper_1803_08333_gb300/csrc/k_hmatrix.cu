@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(HM_THREADS)
 // and a product is the same bits on every run.  Bound: the FP64 pipe (2 lanes per clock and SM, 90 to
 // 93 % busy), 8 multiply-adds per stored entry and column; the FP32 entries are widened with integer
 // operations, which keeps the conversions off that pipe.  Measured on GB300: both products of an
-// ellipsoid of 17280 functions and 11520 cells (47.8 M stored entries), 8 columns: 10.3 ms; one CTA
+// ellipsoid of 17280 functions and 11520 cells (47.8 M stored entries), 8 columns: 10.1 ms; one CTA
 // per block and column with a row a thread and FP64 atomics took 20.2 ms.
 constexpr int HM_COLS = 4;        // columns of a group
 constexpr int HM_TILE = 32;       // rows of a tile (one lane each)
